@@ -44,6 +44,7 @@ struct AdvArgs {
   int rot_safe;                // no stage angle can exceed kRotMax (the host's bound on the
                                // increments; for the double gyre, of nodes in [0, 2] x [0, 1]),
                                // so the steps skip the angle check
+  int dg64;                    // double gyre in double: k_advect_dg64 has taken its nodes
   double p[12];                // flow parameters
   const int32_t* list;         // nullable: process list[0 .. *list_count)
   const unsigned long long* list_count;
@@ -616,6 +617,14 @@ __device__ __forceinline__ bool dg_node_safe(const AdvArgs& a, double x, double 
   return a.rot_safe && x >= 0.0 && x <= 2.0 && y >= 0.0 && y <= 1.0;
 }
 
+// Whether k_advect_dg64 takes a double-gyre node's coordinate z (component p): inside the invariant
+// domain, and zero or far enough from the wall at 0 that a horizon the host allows (dg64_applies)
+// cannot bring it near the end of the float range.  A node is taken when both coordinates are;
+// k_advect integrates the others in double.
+__device__ __forceinline__ bool dg64_coord(double z, int p) {
+  return z == 0.0 || (z >= 0x1p-30 && z <= (p ? 1.0 : 2.0));
+}
+
 // SAFE: the instantiation for AdvArgs::rot_safe (rk4_step's angle-check-free ABC step).  The
 // compensated float kernels are held to five 256-thread blocks per SM (48 registers) for the
 // double gyre (measured on the full mesh: 15.84 ms at 40 registers, six blocks; 15.47 at 48;
@@ -637,7 +646,7 @@ __global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6
   const int lanes = (a.lanes > 0 && a.lanes < (int)blockDim.x) ? a.lanes : (int)blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * lanes; base < count; base += (int64_t)gridDim.x * lanes) {
     const int64_t slot = base + threadIdx.x;
-    const bool active = (int)threadIdx.x < lanes && slot < count;
+    bool active = (int)threadIdx.x < lanes && slot < count;
     const int64_t i = active ? (a.list ? (int64_t)a.list[slot] : slot) : 0;
 
     float xh[DIM], xl[DIM], x0[DIM];
@@ -649,6 +658,12 @@ __global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6
       xh[d] = (float)c;
       xl[d] = (float)(c - (double)xh[d]);
       x0[d] = xh[d];
+    }
+    if constexpr (KIND == FTLE_FLOW_DOUBLE_GYRE && PREC == P64) {
+      if (a.dg64) {  // only the nodes that k_advect_dg64 leaves
+        if (dg64_coord(xd[0], 0) && dg64_coord(xd[1], 1)) active = false;
+        if (!__syncthreads_or(active)) continue;
+      }
     }
     if (a.ckpt && active) store_state<OUT, DIM>(a.ckpt, a.n_mesh, i, xh, xl, xd);
     bool safe_node = false;

@@ -1,0 +1,168 @@
+// Double-precision advection of the 2D double gyre on the FP32 pipes.  GB300 runs a warp's double
+// instruction in about 64 cycles of its SM sub-partition, so k_advect's ~230 double operations per
+// node-step hold the FP64 pipe (18.35 ms for 256 x 128 nodes and 1000 steps, whatever else the
+// kernel does).  Here the state is three floats (72 bits: no rounding of the double state's kind is
+// left in x + dx), the velocity at each stage point is float-float (~2^-47), and the increment
+// h/6 (k1 + 2 k2 + 2 k3 + k4) is formed in float-float with its scale in three parts.  A step's
+// increment is at most ~3e-3 of the domain, so its rounding (~1e-17) sits below half an ulp of the
+// double state (1e-16 for x in [1, 2]) that the double kernel pays at every step.  Measured against
+// an 80-bit RK4 on the 256 x 128 grid: see the figures at launch_advect_dg64.
+//
+// Two lanes per node, as in the float-float re-advection: lane 0 carries x and evaluates
+// (sin, cos)(pi f), lane 1 carries y and evaluates (sin, cos)(pi y); the argument is
+// f = z + a_p z (z - 2) on both, with a_1 = 0.
+#include <math.h>
+
+#include "capi_internal.cuh"
+#include "dsfloat.cuh"
+
+namespace ftle {
+
+constexpr int kDg64Chunk = 1024;  // steps per coefficient table (16 bytes a half step: 32 KB)
+constexpr int kDg64Warps = 8;     // warps per block, at most
+constexpr int kDg64Blocks = 4;    // blocks per SM: 32 warps of 64 registers
+
+// a + (b s + a cm) from a table entry's pair (a, b) and s = sin t, cm = cos t - 1 of a small angle
+// (|t| <= pi/1024): the small terms are summed first, then added to a once.
+__device__ __forceinline__ dsf dg64_turn(float ah, float al, float bh, float bl, float sh, float sl, float cmh,
+                                         float cml) {
+  const float p = __fmul_rn(bh, sh);
+  const float pe = fmaf(bl, sh, fmaf(bh, sl, fmaf(bh, sh, -p)));
+  const float r = fmaf(ah, cmh, p);
+  const float re = fmaf(al, cmh, fmaf(ah, cml, fmaf(ah, cmh, __fsub_rn(p, r))));
+  const dsf v = ds_fast(ah, r);
+  return ds_make(v.h, __fadd_rn(v.l, __fadd_rn(al, __fadd_rn(re, pe))));
+}
+
+// (sin, cos)(pi x) of a float-float x, |x| < 2^12: as ds_sincospi (512 x = j + u, (sin, cos)(pi j/512)
+// from the table, the rest by Taylor) with the period folded into the table index, the integer held
+// in the low bits of the magic-rounded 512 x.  x.h - j/512 is exact.  Error 1.3e-15 rms, 1e-14 at most.
+__device__ __forceinline__ void dg64_sincospi(dsf x, dsf& s, dsf& c) {
+  const float m = fmaf(x.h, 512.0f, kRoundMagic);
+  const float j = __fsub_rn(m, kRoundMagic);
+  const float4 e = __ldg(reinterpret_cast<const float4*>(kDS_SINPI512_TAB) + ((__float_as_int(m) & 1023) ^ 512));
+  // normalized: where 512 x is near j the low part of x would otherwise round the angle at 2^-46
+  const dsf u = ds_fast(fmaf(j, -1.0f / 512.0f, x.h), x.l);
+  const dsf t = ds_mul_u(u, tc<1, true>());
+  const float t2 = t.h * t.h;
+  const dsf su = ds_fast(t.h, fmaf(t.h * t2, fmaf(t2, 1.0f / 120.0f, -1.0f / 6.0f), t.l));
+  const dsf tt = ds_mul_u(t, t);
+  const float cmh = -0.5f * tt.h, cml = fmaf(-0.5f, tt.l, tt.h * tt.h * (1.0f / 24.0f));
+  s = dg64_turn(e.x, e.y, e.z, e.w, su.h, su.l, cmh, cml);
+  c = dg64_turn(e.z, e.w, e.x, e.y, -su.h, -su.l, cmh, cml);
+}
+
+// This lane's velocity component at z without its factor (-pi A, pi A), with the half step's
+// coefficients (a, b = 1 - 2a): sin(pi f) cos(pi y) on lane 0, sin(pi y) cos(pi f) f_x on lane 1.
+__device__ __forceinline__ dsf dg64_vel(int p, const dsf& z, const float4& ab) {
+  const dsf t1 = ds_mul_u(ds_make(p ? 0.f : ab.x, p ? 0.f : ab.y), z);
+  dsf z2 = ds_fast(-2.0f, z.h);  // z - 2, normalized for the nodes near the wall at 2
+  z2 = ds_fast(z2.h, __fadd_rn(z2.l, z.l));
+  const dsf f = ds_add_u(z, ds_mul_u(t1, z2));
+  const dsf fx = ds_add_u(ds_make(2.0f * t1.h, 2.0f * t1.l), ds_make(ab.z, ab.w));
+  const float gh = __shfl_xor_sync(0xffffffffu, fx.h, 1), gl = __shfl_xor_sync(0xffffffffu, fx.l, 1);
+  dsf sn, cs;
+  dg64_sincospi(f, sn, cs);
+  const dsf cq = ds_make(__shfl_xor_sync(0xffffffffu, cs.h, 1), __shfl_xor_sync(0xffffffffu, cs.l, 1));
+  return ds_mul_u(ds_mul_u(sn, cq), ds_make(p ? gh : 1.0f, p ? gl : 0.0f));
+}
+
+template <typename CT>
+__global__ void __launch_bounds__(32 * kDg64Warps, kDg64Blocks) k_advect_dg64(AdvArgs a) {
+  __shared__ float4 s_ab[2 * kDg64Chunk + 1];
+  const int p = threadIdx.x & 1, lane = threadIdx.x & 31;
+  const double scale = (p ? kPi : -kPi) * a.p[0];
+  const dsf S2 = ds_from_double(0.5 * a.h * scale), S1 = ds_from_double(a.h * scale);
+  const double s6 = a.h / 6.0 * scale;
+  const dsf S6 = ds_from_double(s6);
+  const float S6e = (float)(s6 - (double)S6.h - (double)S6.l);
+  const int warps = blockDim.x >> 5;
+  const int64_t tiles = (a.n + 15) / 16;  // 16 nodes per warp
+  const int nchunks = (a.nsteps + kDg64Chunk - 1) / kDg64Chunk;
+  // Tiles go to the blocks in turn, warp by warp, so the SMs' loads differ by one warp; every
+  // warp of a block makes the same number of rounds (the table's barriers are inside them).
+  const int64_t per_round = (int64_t)gridDim.x * warps;
+  bool table_valid = false;
+  for (int64_t r0 = 0; r0 < tiles; r0 += per_round) {
+    const int64_t tile = r0 + (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int64_t i = tile * 16 + (lane >> 1);
+    const bool in = tile < tiles && i < a.n;
+    double z0 = 0.0;
+    if (in) z0 = load_coord<CT>(a.coords, p * a.n_mesh + i);
+    const bool mine = in && dg64_coord(z0, p);
+    // a node is taken when both of its coordinates are; other nodes' lanes integrate zeros
+    const bool both = (__ballot_sync(0xffffffffu, mine) >> (lane & 30) & 3u) == 3u;
+    if (!both) z0 = 0.0;
+    float xh = (float)z0, xm = (float)(z0 - (double)xh), xe = (float)(z0 - (double)xh - (double)xm);
+    int ck_left = a.ckpt_every, ck_slot = 1;
+    if (a.ckpt && both) reinterpret_cast<double*>(a.ckpt)[p * a.n_mesh + i] = z0;
+    for (int ch = 0; ch < nchunks; ++ch) {
+      const int k0 = ch * kDg64Chunk, k1 = min(a.nsteps, k0 + kDg64Chunk);
+      if (!(table_valid && nchunks == 1)) {
+        __syncthreads();
+        for (int m = threadIdx.x; m <= 2 * (k1 - k0); m += blockDim.x) {
+          const dsf c = ds_from_double(a.p[1] * sin(a.p[2] * (a.t0 + 0.5 * a.h * (double)(2 * k0 + m))));
+          const dsf b = ds_add_f(ds_make(-2.0f * c.h, -2.0f * c.l), 1.0f);
+          s_ab[m] = make_float4(c.h, c.l, b.h, b.l);
+        }
+        __syncthreads();
+        table_valid = true;
+      }
+      if (__ballot_sync(0xffffffffu, both) == 0u) continue;
+      float4 c0 = s_ab[0];
+      for (int k = k0; k < k1; ++k) {
+        const float4 c1 = s_ab[2 * (k - k0) + 1], c2 = s_ab[2 * (k - k0) + 2];
+        const dsf x = ds_make(xh, xm);
+        const dsf w1 = dg64_vel(p, x, c0);
+        const dsf w2 = dg64_vel(p, ds_add_u(x, ds_mul_u(S2, w1)), c1);
+        const dsf w3 = dg64_vel(p, ds_add_u(x, ds_mul_u(S2, w2)), c1);
+        const dsf w4 = dg64_vel(p, ds_add_u(x, ds_mul_u(S1, w3)), c2);
+        c0 = c2;
+        const dsf s23 = ds_add_u(w2, w3);
+        const dsf s = ds_add(ds_add_u(w1, w4), ds_make(2.0f * s23.h, 2.0f * s23.l));
+        // dx = S6 s, and x + dx in three parts (|dx| <= |x|: the velocity vanishes at the walls)
+        const float q = __fmul_rn(S6.h, s.h);
+        float e = fmaf(S6.h, s.h, -q);
+        e = fmaf(S6.h, s.l, fmaf(S6.l, s.h, fmaf(S6e, s.h, e)));
+        float h, e1, m, e2, e3;
+        fast_two_sum(xh, q, h, e1);
+        two_sum(xm, e, m, e2);
+        two_sum(m, e1, m, e3);
+        const float lo = __fadd_rn(xe, __fadd_rn(e2, e3));
+        fast_two_sum(h, m, xh, m);
+        fast_two_sum(m, lo, xm, xe);
+        if (a.ckpt && --ck_left == 0) {
+          ck_left = a.ckpt_every;
+          if (both)
+            reinterpret_cast<double*>(reinterpret_cast<char*>(a.ckpt) + (int64_t)ck_slot * a.ckpt_stride_bytes)
+                [p * a.n_mesh + i] = ((double)xe + (double)xm) + (double)xh;
+          ++ck_slot;
+        }
+      }
+    }
+    if (both) reinterpret_cast<double*>(a.out)[p * a.n_mesh + i] = ((double)xe + (double)xm) + (double)xh;
+  }
+}
+
+int launch_advect_dg64(bool coord64, const AdvArgs& a, cudaStream_t s) {
+  const int64_t sms = device_sm_count() > 0 ? device_sm_count() : 1;
+  const int64_t tiles = (a.n + 15) / 16;
+  // Warps per SM: where they fit at once, as many blocks as that takes, of equal size (256 x 128
+  // nodes: 2048 warps on 152 SMs, two blocks of seven warps each); more nodes than that loop.
+  const int64_t per_sm = (tiles + sms - 1) / sms;
+  int64_t blocks = kDg64Blocks, warps = kDg64Warps;
+  if (per_sm <= kDg64Blocks * kDg64Warps) {
+    blocks = (per_sm + kDg64Warps - 1) / kDg64Warps;
+    warps = (per_sm + blocks - 1) / blocks;
+  }
+  const int64_t need = (tiles + warps - 1) / warps;
+  const int grid = (int)(need < sms * blocks ? need : sms * blocks);
+  if (coord64)
+    k_advect_dg64<double><<<grid, 32 * (int)warps, 0, s>>>(a);
+  else
+    k_advect_dg64<float><<<grid, 32 * (int)warps, 0, s>>>(a);
+  FTLE_LAUNCH_CHECK("k_advect_dg64 launch");
+  return FTLE_OK;
+}
+
+}  // namespace ftle

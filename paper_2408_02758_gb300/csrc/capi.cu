@@ -246,6 +246,18 @@ static bool carry_allowed(const ftle_flow* f, bool unchecked, double angle) {
   return f->kind == FTLE_FLOW_ABC && unchecked && angle <= (double)kCarryAngleMax * (1.0 - 1e-3);
 }
 
+// Whether k_advect_dg64 may take a double-gyre problem's nodes (those dg64_coord passes): |eps| <= 1
+// and the step's angles within half a radian, so that every stage point stays within reach of its
+// sine table and the domain stays invariant; the velocity's scale well inside the float range; and
+// the horizon short enough (rate L = pi^2 |A| (1 + 2 |eps|) along the walls) that a coordinate of
+// 2^-30 stays above 2^-30 e^-54 = 2^-108, where float-float still holds its 48 bits.
+static bool dg64_applies(const ftle_flow* f, double h, int nsteps) {
+  const double A = fabs(f->p[0]), eps = fabs(f->p[1]);
+  double angle, diff;
+  return rotation_bounds(f, h, &angle, &diff) && angle <= 0.5 && eps <= 1.0 && kPi * A * fabs(h) >= 0x1p-40 &&
+         kPi * kPi * A * (1.0 + 2.0 * eps) * fabs(h) * (double)nsteps <= 54.0;
+}
+
 AdvArgs make_adv_args(const ftle_mesh* m, const ftle_flow* f, double t0, double T, double dt, int nsteps) {
   AdvArgs a;
   memset(&a, 0, sizeof a);
@@ -414,6 +426,11 @@ int run_advect(const ftle_mesh* m, const ftle_flow* fl, double t0, double T, dou
   }
   const int prec = precision == FTLE_PREC_FP64 ? P64 : (precision == FTLE_PREC_FP32 ? P32 : P32C);
   const int out = precision == FTLE_PREC_FP64 ? O64 : (precision == FTLE_PREC_FP32 ? O32 : O32PAIR);
+  if (prec == P64 && fl->kind == FTLE_FLOW_DOUBLE_GYRE && dg64_applies(fl, a.h, nsteps)) {
+    const int rc = launch_advect_dg64(m->coord_fp64 != 0, a, s);
+    if (rc) return rc;
+    a.dg64 = 1;
+  }
   int block = L.advect_block;
   if (prec == P64 && block > 128) block = 128;
   // by default a grid of 8192 / block blocks per SM (32 of 256 threads), more than fit at once:

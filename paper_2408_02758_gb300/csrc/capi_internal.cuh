@@ -63,6 +63,8 @@ int launch_advect_dg(int prec, int out, bool coord64, const AdvArgs& args, int g
                      size_t smem, cudaStream_t stream);
 int launch_advect_abc(int prec, int out, bool coord64, const AdvArgs& args, int grid, int block,
                       size_t smem, cudaStream_t stream);
+// Double-precision advection of the double gyre's nodes in its domain, on the FP32 pipes.
+int launch_advect_dg64(bool coord64, const AdvArgs& args, cudaStream_t s);
 // Run-parallel float-float re-advection of a compensated 2D double-gyre flowmap (needs the run
 // boundary states, args.seg, and nsteps <= kSegMaxSteps); coef_ws: the workspace's table region.
 int launch_refine_runs_dg(bool coord64, const AdvArgs& args, void* coef_ws, int grid, cudaStream_t s);
