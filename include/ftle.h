@@ -72,7 +72,9 @@ typedef enum ftle_flow_kind {
 } ftle_flow_kind;
 
 /* Arithmetic of the path.
- *   FP64:  everything in double.  flowmap: double [dim][n]; ftle_out: double [n].
+ *   FP64:  everything in double, except that the double gyre's nodes in its invariant domain are
+ *          advected by a three-float state and float-float velocities, whose flowmap is closer to
+ *          exact RK4 than double's.  flowmap: double [dim][n]; ftle_out: double [n].
  *   FP32:  plain float RK4 and float gradient.  flowmap: float [dim][n]; ftle_out: float [n].
  *   FP32C: float RK4 stages with a compensated (two-sum) state and velocity evaluated at the
  *          compensated stage point; the flowmap is stored as (hi, lo) float pairs,
