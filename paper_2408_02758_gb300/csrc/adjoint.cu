@@ -159,11 +159,13 @@ __device__ __forceinline__ DgDer dg_derivs32_rot(float piA, float as, float e1, 
 // The sine and cosine take dg_coef's reduction: u = omega t / pi in double, then sinpi and cospi
 // of u - rint(u) in float, so no double transcendental runs (GB300's FP64 rate is low, and every
 // block rebuilds the table for every segment).
+template <int PREC>
 __device__ __forceinline__ void build_adj_table(const AdvArgs& a, float4* tab, int k0, int k1) {
   const double nu = a.p[2] / kPi;
+  const float eps_lo = PREC == P32C ? (float)(a.p[1] - (double)(float)a.p[1]) : 0.0f;
   for (int m = threadIdx.x; m <= 2 * (k1 - k0); m += blockDim.x) {
     const int mm = 2 * k0 + m;
-    const float2 c = dg_coef(a.p[1], nu, a.t0, 0.5 * a.h, mm);
+    const float2 c = dg_coef(a.p[1], eps_lo, nu, a.t0, 0.5 * a.h, mm);
     const double t = a.t0 + 0.5 * a.h * (double)mm;
     const double u = nu * t, k = rint(u);
     float sr, cr;
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adjoint_rk4(AdvArgs a, const floa
   for (int seg = nseg - 1; seg >= 0; --seg) {
     const int k0 = seg * ce, k1 = min(a.nsteps, k0 + ce);
     __syncthreads();
-    build_adj_table(a, tab, k0, k1);
+    build_adj_table<PREC>(a, tab, k0, k1);
     __syncthreads();
     // recompute the segment's states from its checkpoint with the forward step
     float xh[2] = {0.f, 0.f}, xl[2] = {0.f, 0.f};
@@ -225,7 +227,20 @@ __global__ void __launch_bounds__(kAdjBlock) k_adjoint_rk4(AdvArgs a, const floa
           rk4_step<FTLE_FLOW_DOUBLE_GYRE, 2, PREC, decltype(unchecked)::value>(a, c0, c1, c2, xh, xl, xd);
         }
       };
-      if (safe)
+      if (PREC == P32C && safe && a.dg_carry) {
+        // the forward's carried steps: pairs afresh at the checkpoint and every kDgRefresh steps
+        DgNodes<1> nd;
+        nd.set(0, xh, xl);
+        for (int k = k0; k < k1; ++k) {
+          states[(k - k0) * blockDim.x + threadIdx.x] = make_float2(nd.xh[0], nd.xh[1]);
+          const int m = 2 * (k - k0);
+          if (k == k0)
+            nd.fresh(tab[m].x);
+          else
+            dg_begin_step(nd, k, tab[m].x);
+          nd.step(a, tab[m].x, tab[m + 1].x, tab[m + 2].x);
+        }
+      } else if (safe)
         recompute(std::true_type{});
       else
         recompute(std::false_type{});

@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "dsfloat.cuh"
 
 namespace ftle {
 
@@ -35,6 +36,11 @@ struct AdvArgs {
                                // the steps
   float h6_lo;                 // the same residual for h6_32
   float hs_pi[2];              // double gyre: pi (h/2, h) pi A, the y angle per unit of carried v
+  float hx_pi[3], hx_pi_lo;    // double gyre: -pi (h/2, h, h/6) pi A, pi times the x increment per
+                               // unit of carried u; the last in two parts
+  float hs_pi6, hs_pi6_lo;     // pi h/6 pi A in two parts, the y angle of the whole step
+  int dg_carry;                // double gyre: rot_safe and the step's angles within kCarryAngleMax, so
+                               // the sines and cosines may be carried (dg_step_carried)
   float habc[3][3];            // ABC: (h/2, h, h/6) times (A, B, C), rounded once
   int abc_refresh;             // compensated ABC, unchecked steps: stage one's sines and cosines
                                // evaluated afresh every abc_refresh steps (a power of two),
@@ -492,6 +498,273 @@ __device__ __forceinline__ void abc_steps_carried(const AdvArgs& a, int& k, int 
   }
 }
 
+// The double gyre's (sin, cos) of pi f and pi y at the state, carried from step to step by the unchecked
+// compensated step as base pairs s = (sin pi f, sin pi y) and c (the cosines) and corrections es and
+// ec to them.  Evaluating the pairs afresh takes half of a step's issue slots (two compensated
+// sincospi, the error-free f, and the quarter turns' integer work beside the FP32 pipe).  Carried,
+// stage four's turn adds to the corrections; the state's increment goes beyond stage four's point
+// by a third-order rest, whose first-order turn completes the step's.  The base stays, so that a
+// step's turn is rounded at the corrections' size, not at the pairs', and the angle of the whole
+// step is formed to float's relative rounding with the step scales in two parts (a one-part scale's
+// bias would add up over the steps).  Every kDgRefresh steps the base is taken afresh from a sine
+// table at the state, the turn from the table's angle the first correction.  Emulated on 6000 nodes against
+// an 80-bit RK4 (T = 15, flowmap error of x: rms, median, p99): pairs evaluated at every step
+// 1.7e-7, 5.1e-9, 1.5e-7; carried, refreshed every 8 steps 1.1e-7, 3.8e-9, 1.1e-7; 16: 1.3e-7,
+// 4.0e-9, 1.1e-7 (3.8e-9, 1.0e-7 with the corrections joined to the base halfway, dg_round); 24:
+// 1.8e-7, 5.4e-9, 1.3e-7; without corrections (pairs rounded at every step) every 4: 5.5e-7, 2.1e-8,
+// 5.2e-7.  FTLE of the whole 2048 x 1024 mesh, relative error (max, p99, median): 9.4e-5, 7.5e-6,
+// 2.7e-7 evaluated at every step, 7.6e-5, 6.8e-6, 2.4e-7 carried; refreshed every 8 steps 7.7e-5,
+// 6.5e-6, 2.4e-7 at 11.23 ms instead of 11.01.
+struct DgCarry {
+  float2 s, c, es, ec;
+};
+constexpr int kDgRefresh = 16;  // a power of two
+constexpr int kDgRound = 8;     // a power of two; the corrections join the base every kDgRound steps
+
+// Base and corrections of one component at the argument ah + al (in units of pi): the table's sine and
+// cosine at the nearest multiple of pi/512, and their turn by the rest (at most pi/1024) to third
+// order.  Base plus corrections are the sine and cosine to about 2e-10.
+__device__ __forceinline__ void dg_fresh_pair(float ah, float al, float& s, float& c, float& es, float& ec) {
+  const float kPiF = 3.14159265358979323846f;
+  const float m = fmaf(ah, 512.0f, kRoundMagic);  // the integer sits in its low bits
+  const float4 e = __ldg(reinterpret_cast<const float4*>(kDS_SINPI512_TAB) + ((__float_as_int(m) & 1023) ^ 512));
+  const float t = kPiF * (fmaf(__fsub_rn(m, kRoundMagic), -1.0f / 512.0f, ah) + al);
+  const float t2 = t * t, st = fmaf(t * t2, -1.0f / 6.0f, t), cm = -0.5f * t2;
+  s = e.x;
+  c = e.z;
+  es = fmaf(e.z, st, fmaf(e.x, cm, e.y));
+  ec = fmaf(-e.x, st, fmaf(e.z, cm, e.w));
+}
+
+__device__ __forceinline__ void dg_fresh_pairs(float a, const float* xh, const float* xl, DgCarry& cy) {
+  // f = x + a x (x - 2) at the compensated x, the products error-free
+  float z, zl, fh, fe;
+  fast_two_sum(-2.0f, xh[0], z, zl);
+  const float g = xh[0] * z;
+  const float ge = fmaf(xl[0], fmaf(2.0f, xh[0], -2.0f), fmaf(xh[0], zl, fmaf(xh[0], z, -g)));
+  const float q = a * g;
+  two_sum(xh[0], q, fh, fe);
+  const float fl = fe + (fmaf(a, ge, fmaf(a, g, -q)) + xl[0]);
+  dg_fresh_pair(fh, fl, cy.s.x, cy.c.x, cy.es.x, cy.ec.x);
+  dg_fresh_pair(xh[1], xl[1], cy.s.y, cy.c.y, cy.es.y, cy.ec.y);
+}
+
+// One unchecked step from the carried pairs, with a(t) at the step's start, middle and end.  The
+// stages are those of rk4_step's unchecked step with the x increments scaled by pi (dx) and the
+// slope 1 + 2 a_s (x + dx / pi - 1) formed as W_s + (a_s / pi) dx.
+__device__ __forceinline__ void dg_step_carried(const AdvArgs& a, float a0, float a1, float a2, float* xh, float* xl,
+                                                DgCarry& cy) {
+  const float kPiF = 3.14159265358979323846f, kInvPi = 0.318309886183790671538f;
+  const float2 s0 = add2(cy.s, cy.es), c0 = add2(cy.c, cy.ec);
+  const float e1 = fmaf(2.0f, xh[0], -2.0f);  // 2 (x - 1)
+  const float k1u = s0.x * c0.y, k1v = c0.x * s0.y * fmaf(a0, e1, 1.0f);
+  const float g = fmaf(e1, (0.25f * kPiF) * e1, -kPiF);  // pi x (x - 2)
+  const float dg1 = (a1 - a0) * g, dg2 = (a2 - a0) * g;
+  const float b1 = a1 * kInvPi, b2 = a2 * kInvPi;
+  const float W1 = fmaf(a1, e1, 1.0f), W2 = fmaf(a2, e1, 1.0f);
+  // stage two: turn by the half step's angles, corrections kept apart
+  const float dx2 = a.hx_pi[0] * k1u, w2 = fmaf(b1, dx2, W1);
+  const float tf2 = fmaf(dx2, w2, dg1), ty2 = a.hs_pi[0] * k1v;
+  const float2 u2 = make_float2(tf2, ty2);
+  const float2 q2 = mul2(u2, u2), st2 = fma2(mul2(u2, q2), f2(-1.0f / 6.0f), u2), cm2 = mul2(q2, f2(-0.5f));
+  const float2 ds2 = fma2(s0, cm2, mul2(c0, st2)), dc2 = fma2(c0, cm2, mul2(neg2(s0), st2));
+  const float2 s2 = add2(s0, ds2), c2 = add2(c0, dc2);
+  const float k2u = s2.x * c2.y, k2v = c2.x * s2.y * fmaf(b1, dx2, w2);
+  const float dx3 = a.hx_pi[0] * k2u, w3 = fmaf(b1, dx3, W1);
+  const float2 d3 = make_float2(fmaf(dx3, w3, dg1) - tf2, fmaf(a.hs_pi[0], k2v, -ty2));
+  const float2 s3 = add2(s0, fma2(c2, d3, ds2)), c3 = add2(c0, fma2(neg2(s2), d3, dc2));
+  const float k3u = s3.x * c3.y, k3v = c3.x * s3.y * fmaf(b1, dx3, w3);
+  // stage four: the turn joins the corrections
+  const float dx = a.hx_pi[1] * k3u, w = fmaf(b2, dx, W2);
+  const float2 th = make_float2(fmaf(dx, w, dg2), a.hs_pi[1] * k3v);
+  const float2 t2 = mul2(th, th);
+  const float2 st = fma2(mul2(th, t2), f2(-1.0f / 6.0f), th);
+  const float2 cm = mul2(t2, fma2(t2, f2(1.0f / 24.0f), f2(-0.5f)));
+  const float2 ds = fma2(s0, cm, fma2(c0, st, cy.es)), dc = fma2(c0, cm, fma2(neg2(s0), st, cy.ec));
+  const float2 s4 = add2(cy.s, ds), c4 = add2(cy.c, dc);
+  const float fxs = fmaf(b2, dx, w);
+  const float k4u = s4.x * c4.y, k4v = c4.x * s4.y * fxs;
+  const float sum[2] = {fmaf(2.f, k2u + k3u, k1u + k4u), fmaf(2.f, k2v + k3v, k1v + k4v)};
+  // the rest of the step's angles beyond stage four's
+  const float2 r = make_float2(fxs * fmaf(a.hx_pi[2], sum[0], fmaf(a.hx_pi_lo, sum[0], -dx)),
+                               fmaf(a.hs_pi6, sum[1], fmaf(a.hs_pi6_lo, sum[1], -th.y)));
+  cy.es = fma2(c4, r, ds);
+  cy.ec = fma2(neg2(s4), r, dc);
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    float s, e;
+    comp_add<FTLE_FLOW_DOUBLE_GYRE>(xh[d], fmaf(a.hs[d][2], sum[d], fmaf(a.hs_lo[d], sum[d], xl[d])), s, e);
+    xh[d] = s;
+    xl[d] = e;
+  }
+}
+
+// The corrections join the base by Fast2Sum (exact where the base is the larger, within an ulp of the
+// correction elsewhere), so that they stay small and are rounded accordingly.
+__device__ __forceinline__ void dg_round(float2& b, float2& e) {
+  const float2 s = add2(b, e);
+  e = add2(e, neg2(add2(s, neg2(b))));
+  b = s;
+}
+
+// dg_step_carried of two nodes, one in each lane of every operation (the same bits).  A thread that
+// mixes scalar and paired operations leaves gaps in the FP32 pipe (throttled at 77 % busy, 12.29 ms
+// for the 2048 x 1024 mesh at T = 15); with all of them paired it takes 10.93 ms (15.39 with the pairs
+// evaluated at every step).
+struct DgCarry2 {
+  float2 sf, sy, cf, cy, esf, esy, ecf, ecy;
+};
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return add2(a, neg2(b)); }
+
+__device__ __forceinline__ void dg_step_carried2(const AdvArgs& a, float a0, float a1, float a2, float2* xh, float2* xl,
+                                                 DgCarry2& p) {
+  const float kPiF = 3.14159265358979323846f, kInvPi = 0.318309886183790671538f;
+  const float2 sf = add2(p.sf, p.esf), sy = add2(p.sy, p.esy), cf = add2(p.cf, p.ecf), cy = add2(p.cy, p.ecy);
+  const float2 one = f2(1.0f), A1 = f2(a1), A2 = f2(a2);
+  const float2 e1 = fma2(f2(2.0f), xh[0], f2(-2.0f));
+  const float2 k1u = mul2(sf, cy), k1v = mul2(mul2(cf, sy), fma2(f2(a0), e1, one));
+  const float2 g = fma2(e1, mul2(f2(0.25f * kPiF), e1), f2(-kPiF));
+  const float2 dg1 = mul2(f2(a1 - a0), g), dg2 = mul2(f2(a2 - a0), g);
+  const float2 b1 = f2(a1 * kInvPi), b2 = f2(a2 * kInvPi);
+  const float2 W1 = fma2(A1, e1, one), W2 = fma2(A2, e1, one);
+  const float2 m6 = f2(-1.0f / 6.0f), mh = f2(-0.5f);
+  // stage two
+  const float2 hx = f2(a.hx_pi[0]), hy = f2(a.hs_pi[0]);
+  const float2 dx2 = mul2(hx, k1u), w2 = fma2(b1, dx2, W1);
+  const float2 tf2 = fma2(dx2, w2, dg1), ty2 = mul2(hy, k1v);
+  const float2 qf = mul2(tf2, tf2), qy = mul2(ty2, ty2);
+  const float2 stf = fma2(mul2(tf2, qf), m6, tf2), sty = fma2(mul2(ty2, qy), m6, ty2);
+  const float2 cmf = mul2(qf, mh), cmy = mul2(qy, mh);
+  const float2 dsf = fma2(sf, cmf, mul2(cf, stf)), dcf = fma2(cf, cmf, mul2(neg2(sf), stf));
+  const float2 dsy = fma2(sy, cmy, mul2(cy, sty)), dcy = fma2(cy, cmy, mul2(neg2(sy), sty));
+  const float2 sf2 = add2(sf, dsf), cf2 = add2(cf, dcf), sy2 = add2(sy, dsy), cy2 = add2(cy, dcy);
+  const float2 k2u = mul2(sf2, cy2), k2v = mul2(mul2(cf2, sy2), fma2(b1, dx2, w2));
+  // stage three
+  const float2 dx3 = mul2(hx, k2u), w3 = fma2(b1, dx3, W1);
+  const float2 df = sub2(fma2(dx3, w3, dg1), tf2), dy = fma2(hy, k2v, neg2(ty2));
+  const float2 sf3 = add2(sf, fma2(cf2, df, dsf)), cf3 = add2(cf, fma2(neg2(sf2), df, dcf));
+  const float2 sy3 = add2(sy, fma2(cy2, dy, dsy)), cy3 = add2(cy, fma2(neg2(sy2), dy, dcy));
+  const float2 k3u = mul2(sf3, cy3), k3v = mul2(mul2(cf3, sy3), fma2(b1, dx3, w3));
+  // stage four
+  const float2 dx = mul2(f2(a.hx_pi[1]), k3u), w = fma2(b2, dx, W2);
+  const float2 tf = fma2(dx, w, dg2), ty = mul2(f2(a.hs_pi[1]), k3v);
+  const float2 uf = mul2(tf, tf), uy = mul2(ty, ty);
+  const float2 vf = fma2(mul2(tf, uf), m6, tf), vy = fma2(mul2(ty, uy), m6, ty);
+  const float2 mf = mul2(uf, fma2(uf, f2(1.0f / 24.0f), mh)), my = mul2(uy, fma2(uy, f2(1.0f / 24.0f), mh));
+  const float2 esf = fma2(sf, mf, fma2(cf, vf, p.esf)), ecf = fma2(cf, mf, fma2(neg2(sf), vf, p.ecf));
+  const float2 esy = fma2(sy, my, fma2(cy, vy, p.esy)), ecy = fma2(cy, my, fma2(neg2(sy), vy, p.ecy));
+  const float2 sf4 = add2(p.sf, esf), cf4 = add2(p.cf, ecf), sy4 = add2(p.sy, esy), cy4 = add2(p.cy, ecy);
+  const float2 fxs = fma2(b2, dx, w);
+  const float2 k4u = mul2(sf4, cy4), k4v = mul2(mul2(cf4, sy4), fxs);
+  const float2 su = fma2(f2(2.f), add2(k2u, k3u), add2(k1u, k4u)), sv = fma2(f2(2.f), add2(k2v, k3v), add2(k1v, k4v));
+  const float2 rf = mul2(fxs, fma2(f2(a.hx_pi[2]), su, fma2(f2(a.hx_pi_lo), su, neg2(dx))));
+  const float2 ry = fma2(f2(a.hs_pi6), sv, fma2(f2(a.hs_pi6_lo), sv, neg2(ty)));
+  p.esf = fma2(cf4, rf, esf);
+  p.ecf = fma2(neg2(sf4), rf, ecf);
+  p.esy = fma2(cy4, ry, esy);
+  p.ecy = fma2(neg2(sy4), ry, ecy);
+  // the compensated state: fast_two_sum of both nodes
+  const float2 iu = fma2(f2(a.hs[0][2]), su, fma2(f2(a.hs_lo[0]), su, xl[0]));
+  const float2 iv = fma2(f2(a.hs[1][2]), sv, fma2(f2(a.hs_lo[1]), sv, xl[1]));
+  const float2 nx = add2(xh[0], iu), ny = add2(xh[1], iv);
+  xl[0] = sub2(iu, sub2(nx, xh[0]));
+  xl[1] = sub2(iv, sub2(ny, xh[1]));
+  xh[0] = nx;
+  xh[1] = ny;
+}
+
+// A step of one node or of two.
+template <int N>
+struct DgNodes;
+template <>
+struct DgNodes<1> {
+  float xh[2], xl[2];
+  DgCarry c;
+  __device__ __forceinline__ void fresh(float a) { dg_fresh_pairs(a, xh, xl, c); }
+  __device__ __forceinline__ void round() {
+    dg_round(c.s, c.es);
+    dg_round(c.c, c.ec);
+  }
+  __device__ __forceinline__ void step(const AdvArgs& a, float a0, float a1, float a2) {
+    dg_step_carried(a, a0, a1, a2, xh, xl, c);
+  }
+  __device__ __forceinline__ void get(int, float* h, float* l) const { h[0] = xh[0], h[1] = xh[1], l[0] = xl[0], l[1] = xl[1]; }
+  __device__ __forceinline__ void set(int, const float* h, const float* l) { xh[0] = h[0], xh[1] = h[1], xl[0] = l[0], xl[1] = l[1]; }
+};
+template <>
+struct DgNodes<2> {
+  float2 xh[2], xl[2];
+  DgCarry2 c;
+  __device__ __forceinline__ void get(int q, float* h, float* l) const {
+#pragma unroll
+    for (int d = 0; d < 2; ++d) h[d] = q ? xh[d].y : xh[d].x, l[d] = q ? xl[d].y : xl[d].x;
+  }
+  __device__ __forceinline__ void set(int q, const float* h, const float* l) {
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      if (q)
+        xh[d].y = h[d], xl[d].y = l[d];
+      else
+        xh[d].x = h[d], xl[d].x = l[d];
+    }
+  }
+  __device__ __forceinline__ void fresh(float a) {
+    float h[2], l[2];
+    DgCarry u, v;
+    get(0, h, l);
+    dg_fresh_pairs(a, h, l, u);
+    get(1, h, l);
+    dg_fresh_pairs(a, h, l, v);
+    c.sf = make_float2(u.s.x, v.s.x), c.sy = make_float2(u.s.y, v.s.y);
+    c.cf = make_float2(u.c.x, v.c.x), c.cy = make_float2(u.c.y, v.c.y);
+    c.esf = make_float2(u.es.x, v.es.x), c.esy = make_float2(u.es.y, v.es.y);
+    c.ecf = make_float2(u.ec.x, v.ec.x), c.ecy = make_float2(u.ec.y, v.ec.y);
+  }
+  __device__ __forceinline__ void round() {
+    dg_round(c.sf, c.esf);
+    dg_round(c.sy, c.esy);
+    dg_round(c.cf, c.ecf);
+    dg_round(c.cy, c.ecy);
+  }
+  __device__ __forceinline__ void step(const AdvArgs& a, float a0, float a1, float a2) {
+    dg_step_carried2(a, a0, a1, a2, xh, xl, c);
+  }
+};
+
+// What step k (any multiple of kDgRound) begins with.
+template <int N>
+__device__ __forceinline__ void dg_begin_step(DgNodes<N>& nd, int k, float a) {
+  if ((k & (kDgRefresh - 1)) == 0)
+    nd.fresh(a);
+  else if ((k & (kDgRound - 1)) == 0)
+    nd.round();
+}
+
+// Steps k .. stop - 1 from the carried pairs (k ends at stop); at(m): a(t) at half step m.  Whole
+// periods are unrolled by two: the loop's own work is a tenth of a step's issue slots.
+template <int N, class At>
+__device__ __forceinline__ void dg_steps_carried(const AdvArgs& a, int& k, int stop, DgNodes<N>& nd, At at) {
+  while (k < stop) {
+    float a0 = at(2 * k);
+    dg_begin_step(nd, k, a0);
+    const int g = min(stop, (k | (kDgRound - 1)) + 1);
+    auto one = [&](int q) {
+      const float a2 = at(2 * q + 2);
+      nd.step(a, a0, at(2 * q + 1), a2);
+      a0 = a2;
+    };
+    if (g - k == kDgRound) {
+#pragma unroll 2
+      for (int q = 0; q < kDgRound; ++q) one(k + q);
+      k = g;
+    } else {
+#pragma unroll 1
+      for (; k < g; ++k) one(k);
+    }
+  }
+}
+
 // Advance one node by one classic RK4 step (stages at t, t + h/2, t + h/2, t + h, with the
 // coefficients c0, c1, c2 of those half steps).  P64 updates xd; P32 updates xh; P32C updates
 // the compensated pair (xh, xl), evaluating the velocity at compensated stage points.  SAFE
@@ -584,11 +857,12 @@ template <int KIND, int PREC>
 __device__ __forceinline__ void build_table(const AdvArgs& a, float2* tab32, double* tab64, int k0, int k1) {
   if constexpr (KIND == FTLE_FLOW_DOUBLE_GYRE) {
     const double nu = a.p[2] / kPi;  // omega / pi
+    const float eps_lo = PREC == P32C ? (float)(a.p[1] - (double)(float)a.p[1]) : 0.0f;
     for (int m = threadIdx.x; m <= 2 * (k1 - k0); m += blockDim.x) {
       if constexpr (PREC == P64) {
         tab64[m] = sin(a.p[2] * (a.t0 + 0.5 * a.h * (double)(2 * k0 + m)));
       } else {
-        tab32[m] = dg_coef(a.p[1], nu, a.t0, 0.5 * a.h, 2 * k0 + m);
+        tab32[m] = dg_coef(a.p[1], eps_lo, nu, a.t0, 0.5 * a.h, 2 * k0 + m);
       }
     }
   }
@@ -633,7 +907,7 @@ __device__ __forceinline__ bool dg64_coord(double z, int p) {
 // CARRY (with SAFE, the compensated ABC step): stage one's (sin, cos) carried across steps
 // (abc_step_carried, AdvArgs::abc_refresh > 1).
 template <int KIND, int DIM, int PREC, int OUT, typename CT, bool SAFE = false, bool CARRY = false>
-__global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6 : 5) : 1) k_advect(AdvArgs a) {
+__global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6 : 4) : 1) k_advect(AdvArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr bool kTable = (KIND == FTLE_FLOW_DOUBLE_GYRE);
   float2* tab32 = reinterpret_cast<float2*>(smem_raw);
@@ -748,6 +1022,175 @@ __global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6
         if (a.rec) store_record<DIM>(a.rec, i, x0, xh, xl);
       }
     }
+  }
+}
+
+// Compensated double-gyre advection where the steps carry the sines and cosines (AdvArgs::dg_carry),
+// up to two nodes per thread: nodes i + q * stride, q < count.  Safe nodes (dg_node_safe) take the
+// carried steps, two at a time where both are safe; the others take rk4_step's checked step.  tab:
+// the coefficient table of steps k0 .. k1; at() and coef() read it.
+template <int N>
+struct DgWalk {
+  DgNodes<N> nd;
+  float x0[N][2];
+  int ck_left, ck_slot, seg_slot, next_seg;
+
+  // (ok: the thread's nodes inside the mesh; inside chunk() all of them are)
+  __device__ __forceinline__ void store(const AdvArgs& a, void* base, int64_t i, int64_t stride,
+                                        const bool* ok = nullptr) const {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      if (ok && !ok[q]) continue;
+      float h[2], l[2];
+      nd.get(q, h, l);
+      store_state<O32PAIR, 2>(base, a.n_mesh, i + q * stride, h, l, nullptr);
+    }
+  }
+  __device__ __forceinline__ void begin(const AdvArgs& a, int64_t i, int64_t stride, const float (*h)[2],
+                                        const float (*l)[2], const bool* ok) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      nd.set(q, h[q], l[q]);
+      x0[q][0] = h[q][0], x0[q][1] = h[q][1];
+    }
+    ck_left = a.ckpt_every, ck_slot = 1, seg_slot = 0, next_seg = a.seg_len;
+    if (a.ckpt) store(a, a.ckpt, i, stride, ok);
+  }
+  // Steps k0 .. k1 - 1, storing checkpoints and run-boundary states on the way.
+  template <bool CARRY, bool SAFE>
+  __device__ __forceinline__ void chunk(const AdvArgs& a, const float2* tab, int k0, int k1, int64_t i, int64_t stride) {
+    auto at = [&](int m) { return tab[m - 2 * k0].x; };
+    for (int k = k0; k < k1;) {
+      int to = a.seg ? min(k1, next_seg) : k1;
+      if (a.ckpt) to = min(to, k + ck_left);
+      const int from = k;
+      if constexpr (CARRY) {
+        dg_steps_carried<N>(a, k, to, nd, at);
+      } else {
+        float h[2], l[2];
+        nd.get(0, h, l);
+        for (; k < to; ++k) {
+          const int m = 2 * (k - k0);
+          rk4_step<FTLE_FLOW_DOUBLE_GYRE, 2, P32C, SAFE>(a, coef_at<FTLE_FLOW_DOUBLE_GYRE, P32C>(tab, nullptr, m),
+                                                         coef_at<FTLE_FLOW_DOUBLE_GYRE, P32C>(tab, nullptr, m + 1),
+                                                         coef_at<FTLE_FLOW_DOUBLE_GYRE, P32C>(tab, nullptr, m + 2), h, l,
+                                                         nullptr);
+        }
+        nd.set(0, h, l);
+      }
+      ck_left -= k - from;
+      if (a.ckpt && ck_left == 0) {
+        ck_left = a.ckpt_every;
+        store(a, reinterpret_cast<char*>(a.ckpt) + (int64_t)ck_slot * a.ckpt_stride_bytes, i, stride);
+        ++ck_slot;
+        // the adjoint recomputes from here, so the pairs start afresh
+        if constexpr (CARRY)
+          if (k & (kDgRefresh - 1)) nd.fresh(at(2 * k));
+      }
+      if (a.seg && k == next_seg) {
+        if (seg_slot < kSegments - 1) store(a, a.seg + (int64_t)seg_slot * a.seg_stride, i, stride);
+        ++seg_slot;
+        next_seg += a.seg_len;
+      }
+    }
+  }
+  __device__ __forceinline__ void end(const AdvArgs& a, int64_t i, int64_t stride, const bool* ok) {
+    if (a.seg)  // boundaries at or past the last step hold the final state
+      for (; seg_slot < kSegments - 1; ++seg_slot) store(a, a.seg + (int64_t)seg_slot * a.seg_stride, i, stride, ok);
+    store(a, a.out, i, stride, ok);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      if (!ok[q]) continue;
+      float h[2], l[2];
+      nd.get(q, h, l);
+      if (a.rec) store_record<2>(a.rec, i + q * stride, x0[q], h, l);
+    }
+  }
+};
+
+// One chunk of steps of a thread's N nodes: two at a time where both are safe (dg_node_safe), else node
+// by node, the unsafe ones by rk4_step's checked step.  A chunk starts at a multiple of kDgRefresh,
+// so no pairs pass from one to the next.
+template <int N>
+__device__ __forceinline__ void dg_walk_chunk(const AdvArgs& a, const float2* tab, int k0, int k1, int64_t i,
+                                              int64_t stride, const bool* active, const bool* safe, DgWalk<N>& w) {
+  static_assert(kAdvChunk % kDgRefresh == 0, "a chunk starts with fresh pairs");
+  if (N == 2 && active[0] && active[N - 1] && safe[0] && safe[N - 1]) {
+    w.template chunk<true, true>(a, tab, k0, k1, i, stride);
+    return;
+  }
+  const int ck_left = w.ck_left, ck_slot = w.ck_slot, seg_slot = w.seg_slot, next_seg = w.next_seg;
+#pragma unroll 1
+  for (int q = 0; q < N; ++q) {
+    if (!active[q]) continue;
+    DgWalk<1> v;
+    float h[2], l[2];
+    w.nd.get(q, h, l);
+    v.nd.set(0, h, l);
+    v.ck_left = ck_left, v.ck_slot = ck_slot, v.seg_slot = seg_slot, v.next_seg = next_seg;
+    if (safe[q])
+      v.template chunk<true, true>(a, tab, k0, k1, i + q * stride, 0);
+    else
+      v.template chunk<false, false>(a, tab, k0, k1, i + q * stride, 0);
+    v.nd.get(0, h, l);
+    w.nd.set(q, h, l);
+    w.ck_left = v.ck_left, w.ck_slot = v.ck_slot, w.seg_slot = v.seg_slot, w.next_seg = v.next_seg;
+  }
+}
+
+// A thread's N nodes i + q * stride, from their coordinates to their records, in a block that shares
+// the coefficient table.  build(k0, k1) makes the table of a chunk (whole block; every thread calls
+// dg_walk), or returns at once when it is there already.
+template <int N, typename CT, class Build>
+__device__ __forceinline__ void dg_walk(const AdvArgs& a, const float2* tab, int64_t i, int64_t stride, int64_t end,
+                                        Build build) {
+  bool active[N], safe[N], any = false;
+  float h[N][2], l[N][2];
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    active[q] = i + q * stride < end;
+    any = any || active[q];
+    double x[2];
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      x[d] = active[q] ? load_coord<CT>(a.coords, d * a.n_mesh + i + q * stride) : 0.0;
+      h[q][d] = (float)x[d];
+      l[q][d] = (float)(x[d] - (double)h[q][d]);
+    }
+    safe[q] = dg_node_safe(a, x[0], x[1]);
+  }
+  DgWalk<N> w;
+  w.begin(a, i, stride, h, l, active);
+  for (int k0 = 0; k0 < a.nsteps; k0 += kAdvChunk) {
+    const int k1 = min(a.nsteps, k0 + kAdvChunk);
+    build(k0, k1);
+    if (any) dg_walk_chunk<N>(a, tab, k0, k1, i, stride, active, safe, w);
+  }
+  w.end(a, i, stride, active);
+}
+
+// k_advect for compensated double-gyre flowmaps whose steps carry the sines and cosines: N nodes per
+// thread, 32 N consecutive nodes per warp.  Rounds of tiles go to the blocks in turn, warp by warp.
+template <int N>
+constexpr int kDgBlocks = N == 2 ? 2 : 4;  // 256-thread blocks per SM: 128 or 64 registers
+
+template <int N, typename CT>
+__global__ void __launch_bounds__(256, kDgBlocks<N>) k_advect_dg(AdvArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* tab = reinterpret_cast<float2*>(smem_raw);
+  const int warps = blockDim.x >> 5;
+  const int64_t tiles = (a.n + 32 * N - 1) / (32 * N), per_round = (int64_t)gridDim.x * warps;
+  bool valid = false;
+  auto build = [&](int k0, int k1) {
+    if (valid && a.nsteps <= kAdvChunk) return;
+    __syncthreads();
+    build_table<FTLE_FLOW_DOUBLE_GYRE, P32C>(a, tab, nullptr, k0, k1);
+    __syncthreads();
+    valid = true;
+  };
+  for (int64_t r0 = 0; r0 < tiles; r0 += per_round) {  // the same rounds for every warp of the block
+    const int64_t tile = r0 + (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    dg_walk<N, CT>(a, tab, tile * 32 * N + (threadIdx.x & 31), 32, a.n, build);
   }
 }
 

@@ -25,36 +25,6 @@ constexpr int kDg64Chunk = 1024;  // steps per coefficient table (16 bytes a hal
 constexpr int kDg64Warps = 8;     // warps per block, at most
 constexpr int kDg64Blocks = 4;    // blocks per SM: 32 warps of 64 registers
 
-// a + (b s + a cm) from a table entry's pair (a, b) and s = sin t, cm = cos t - 1 of a small angle
-// (|t| <= pi/1024): the small terms are summed first, then added to a once.
-__device__ __forceinline__ dsf dg64_turn(float ah, float al, float bh, float bl, float sh, float sl, float cmh,
-                                         float cml) {
-  const float p = __fmul_rn(bh, sh);
-  const float pe = fmaf(bl, sh, fmaf(bh, sl, fmaf(bh, sh, -p)));
-  const float r = fmaf(ah, cmh, p);
-  const float re = fmaf(al, cmh, fmaf(ah, cml, fmaf(ah, cmh, __fsub_rn(p, r))));
-  const dsf v = ds_fast(ah, r);
-  return ds_make(v.h, __fadd_rn(v.l, __fadd_rn(al, __fadd_rn(re, pe))));
-}
-
-// (sin, cos)(pi x) of a float-float x, |x| < 2^12: as ds_sincospi (512 x = j + u, (sin, cos)(pi j/512)
-// from the table, the rest by Taylor) with the period folded into the table index, the integer held
-// in the low bits of the magic-rounded 512 x.  x.h - j/512 is exact.  Error 1.3e-15 rms, 1e-14 at most.
-__device__ __forceinline__ void dg64_sincospi(dsf x, dsf& s, dsf& c) {
-  const float m = fmaf(x.h, 512.0f, kRoundMagic);
-  const float j = __fsub_rn(m, kRoundMagic);
-  const float4 e = __ldg(reinterpret_cast<const float4*>(kDS_SINPI512_TAB) + ((__float_as_int(m) & 1023) ^ 512));
-  // normalized: where 512 x is near j the low part of x would otherwise round the angle at 2^-46
-  const dsf u = ds_fast(fmaf(j, -1.0f / 512.0f, x.h), x.l);
-  const dsf t = ds_mul_u(u, tc<1, true>());
-  const float t2 = t.h * t.h;
-  const dsf su = ds_fast(t.h, fmaf(t.h * t2, fmaf(t2, 1.0f / 120.0f, -1.0f / 6.0f), t.l));
-  const dsf tt = ds_mul_u(t, t);
-  const float cmh = -0.5f * tt.h, cml = fmaf(-0.5f, tt.l, tt.h * tt.h * (1.0f / 24.0f));
-  s = dg64_turn(e.x, e.y, e.z, e.w, su.h, su.l, cmh, cml);
-  c = dg64_turn(e.z, e.w, e.x, e.y, -su.h, -su.l, cmh, cml);
-}
-
 // This lane's velocity component at z without its factor (-pi A, pi A), with the half step's
 // coefficients (a, b = 1 - 2a): sin(pi f) cos(pi y) on lane 0, sin(pi y) cos(pi f) f_x on lane 1.
 __device__ __forceinline__ dsf dg64_vel(int p, const dsf& z, const float4& ab) {
@@ -65,7 +35,7 @@ __device__ __forceinline__ dsf dg64_vel(int p, const dsf& z, const float4& ab) {
   const dsf fx = ds_add_u(ds_make(2.0f * t1.h, 2.0f * t1.l), ds_make(ab.z, ab.w));
   const float gh = __shfl_xor_sync(0xffffffffu, fx.h, 1), gl = __shfl_xor_sync(0xffffffffu, fx.l, 1);
   dsf sn, cs;
-  dg64_sincospi(f, sn, cs);
+  ds_sincospi_fold(f, sn, cs);
   const dsf cq = ds_make(__shfl_xor_sync(0xffffffffu, cs.h, 1), __shfl_xor_sync(0xffffffffu, cs.l, 1));
   return ds_mul_u(ds_mul_u(sn, cq), ds_make(p ? gh : 1.0f, p ? gl : 0.0f));
 }

@@ -127,6 +127,35 @@ __global__ void __launch_bounds__(256, PREC == P32C ? 4 : 1) k_batch_advect(cons
   }
 }
 
+// The items of instances whose double-gyre steps carry the sines and cosines (AdvArgs::dg_carry): as
+// k_advect_dg (the same steps, the same bits), two nodes per thread, an item's nodes in its warps'
+// order.
+__global__ void __launch_bounds__(256, kDgBlocks<2>) k_batch_advect_dg(const BatchInst* __restrict__ insts,
+                                                                       const BatchItem* __restrict__ items, int n_items,
+                                                                       unsigned int* next) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* tab = reinterpret_cast<float2*>(smem_raw);
+  __shared__ int s_item, s_tab_inst;
+  if (threadIdx.x == 0) s_tab_inst = -1;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= n_items) break;
+    const BatchItem item = items[it];
+    const AdvArgs a = insts[item.inst].adv;
+    auto build = [&](int k0, int k1) {
+      if (s_tab_inst == item.inst && a.nsteps <= kAdvChunk) return;
+      __syncthreads();
+      build_table<FTLE_FLOW_DOUBLE_GYRE, P32C>(a, tab, nullptr, k0, k1);
+      if (threadIdx.x == 0) s_tab_inst = item.inst;
+      __syncthreads();
+    };
+    dg_walk<2, float>(a, tab, (int64_t)item.lo + (threadIdx.x >> 5) * 64 + (threadIdx.x & 31), 32, item.hi, build);
+  }
+}
+
 template <int DIM, int PL>
 __global__ void __launch_bounds__(256) k_batch_grad(const BatchInst* __restrict__ insts,
                                                     const BatchItem* __restrict__ items, int n_items,
@@ -252,6 +281,13 @@ int launch_batch_mark(const BatchInst* insts, const int2* flags, const unsigned 
   return FTLE_OK;
 }
 
+static int launch_batch_advect_dg(const BatchInst* insts, const BatchItem* items, int n_items, unsigned int* next, int grid,
+                                  int block, size_t smem, cudaStream_t s) {
+  k_batch_advect_dg<<<grid, block, smem, s>>>(insts, items, n_items, next);
+  FTLE_LAUNCH_CHECK("k_batch_advect_dg launch");
+  return FTLE_OK;
+}
+
 // ------------------------------------------------------------------------------- planning
 
 namespace {
@@ -306,6 +342,9 @@ struct BatchPlanHost {
   BatchLayout L;
   std::vector<BatchInst> insts;
   std::vector<BatchItem> adv_items, grad_items;
+  int carry_block = 128;  // threads per block of k_batch_advect_dg
+  int n_carry = 0;  // the first adv_items: carried double-gyre steps (k_batch_advect_dg)
+  int max_steps_carry = 0;
 };
 
 int plan_batch(int32_t n_inst, const ftle_mesh* meshes, const ftle_flow* flows, const double* T, double dt,
@@ -334,6 +373,9 @@ int plan_batch(int32_t n_inst, const ftle_mesh* meshes, const ftle_flow* flows, 
   P.ws = reinterpret_cast<char*>(workspace);
   // launch shapes (tile of the gradient queue: opt->grad_tile, a multiple of the block)
   P.adv_block = Lc.advect_block;
+  // four warps: 256-node items, finer than a block of eight for the last round (two 512 x 256
+  // instances: 1201 us a call against 1313; 24 uneven instances: the same)
+  P.carry_block = Lc.advect_shape ? Lc.advect_block : 128;
   P.grad_block = Lc.grad_block;
   P.grad_tile = (opt && opt->grad_tile > 0) ? opt->grad_tile : Lc.grad_block;
   if (P.grad_tile % P.grad_block) return fail(FTLE_EINVAL, "batch: grad_tile must be a multiple of grad_block");
@@ -373,13 +415,23 @@ int plan_batch(int32_t n_inst, const ftle_mesh* meshes, const ftle_flow* flows, 
     bi.off = off;
     off += meshes[q].n_nodes;
   }
-  // advection queue: items of one block of nodes, longest (steps x nodes) first
-  for (int q = 0; q < n_inst; ++q)
-    for (int64_t lo = 0; lo < meshes[q].n_nodes; lo += P.adv_block)
-      P.adv_items.push_back({q, (int32_t)lo, (int32_t)std::min<int64_t>(meshes[q].n_nodes, lo + P.adv_block), 0});
-  std::stable_sort(P.adv_items.begin(), P.adv_items.end(), [&](const BatchItem& x, const BatchItem& y) {
-    return (int64_t)steps[x.inst] * (x.hi - x.lo) > (int64_t)steps[y.inst] * (y.hi - y.lo);
-  });
+  // advection queues, one after the other: items of instances with carried double-gyre steps (two nodes
+  // per thread), then of the others; each of one block of threads, longest (steps x nodes) first
+  auto carry = [&](int q) { return precision == FTLE_PREC_FP32C && P.insts[q].adv.dg_carry; };
+  for (int pass = 0; pass < 2; ++pass) {
+    const size_t first = P.adv_items.size();
+    for (int q = 0; q < n_inst; ++q) {
+      if (carry(q) != (pass == 0)) continue;
+      if (pass == 0) P.max_steps_carry = std::max(P.max_steps_carry, steps[q]);
+      const int64_t len = pass == 0 ? 2 * P.carry_block : P.adv_block;
+      for (int64_t lo = 0; lo < meshes[q].n_nodes; lo += len)
+        P.adv_items.push_back({q, (int32_t)lo, (int32_t)std::min<int64_t>(meshes[q].n_nodes, lo + len), 0});
+    }
+    std::stable_sort(P.adv_items.begin() + first, P.adv_items.end(), [&](const BatchItem& x, const BatchItem& y) {
+      return (int64_t)steps[x.inst] * (x.hi - x.lo) > (int64_t)steps[y.inst] * (y.hi - y.lo);
+    });
+    if (pass == 0) P.n_carry = (int)P.adv_items.size();
+  }
   for (int q = 0; q < n_inst; ++q)
     for (int64_t lo = 0; lo < meshes[q].n_nodes; lo += P.grad_tile)
       P.grad_items.push_back({q, (int32_t)lo, (int32_t)std::min<int64_t>(meshes[q].n_nodes, lo + P.grad_tile), 0});
@@ -422,15 +474,25 @@ int enqueue_batch(const BatchPlanHost& P, cudaStream_t s) {
   const BatchInst* insts = reinterpret_cast<const BatchInst*>(w + P.L.insts);
   unsigned int* adv_next = reinterpret_cast<unsigned int*>(&hdr->reserved[0]);
   unsigned int* grad_next = reinterpret_cast<unsigned int*>(&hdr->reserved[1]);
+  unsigned int* carry_next = reinterpret_cast<unsigned int*>(&hdr->reserved[2]);
   int2* flags = reinterpret_cast<int2*>(w + P.L.flags);
   int2* marks = reinterpret_cast<int2*>(w + P.L.marks);
   const int sms = device_sm_count() > 0 ? device_sm_count() : 1;
   const int prec = P.precision == FTLE_PREC_FP32C ? P32C : P32;
   const int pl = P.precision == FTLE_PREC_FP32C ? PHI32PAIR : PHI32;
   FTLE_CUDA_CHECK(cudaMemsetAsync(hdr, 0, sizeof(ftle_counters), s));
+  const BatchItem* items = reinterpret_cast<const BatchItem*>(w + P.L.adv_items);
+  const int n_items = (int)P.adv_items.size();
+  if (P.n_carry > 0) {
+    const int grid = std::min(sms * kDgBlocks<2> * 256 / P.carry_block, P.n_carry);  // all resident
+    if ((rc = launch_batch_advect_dg(insts, items, P.n_carry, carry_next, grid, P.carry_block,
+                                     advect_smem_bytes(P.kind, prec, P.max_steps_carry), s)))
+      return rc;
+  }
   const size_t smem = advect_smem_bytes(P.kind, prec, P.max_steps);
-  if ((rc = launch_batch_advect(P.kind, P.dim, prec, insts, reinterpret_cast<const BatchItem*>(w + P.L.adv_items),
-                                (int)P.adv_items.size(), adv_next, P.adv_grid, P.adv_block, smem, s)))
+  if (n_items > P.n_carry &&
+      (rc = launch_batch_advect(P.kind, P.dim, prec, insts, items + P.n_carry, n_items - P.n_carry, adv_next, P.adv_grid,
+                                P.adv_block, smem, s)))
     return rc;
   if ((rc = launch_batch_grad(P.dim, pl, insts, reinterpret_cast<const BatchItem*>(w + P.L.grad_items),
                               (int)P.grad_items.size(), grad_next, hdr, flags, P.grad_grid, P.grad_block, s)))

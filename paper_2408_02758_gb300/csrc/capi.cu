@@ -151,7 +151,10 @@ Launch resolve_launch(const ftle_options* opt) {
   Launch L;
   if (opt) {
     if (opt->refine_kappa != 0.0) L.refine_kappa = opt->refine_kappa;
-    if (opt->advect_block > 0) L.advect_block = opt->advect_block;
+    if (opt->advect_block > 0) {
+      L.advect_block = opt->advect_block;
+      L.advect_shape = true;
+    }
     if (opt->advect_blocks_per_sm > 0) L.advect_bps = opt->advect_blocks_per_sm;
     if (opt->grad_block > 0) L.grad_block = opt->grad_block;
     if (opt->refine_lanes > 0) L.refine_lanes = opt->refine_lanes;
@@ -283,6 +286,13 @@ AdvArgs make_adv_args(const ftle_mesh* m, const ftle_flow* f, double t0, double 
   if (f->kind == FTLE_FLOW_DOUBLE_GYRE) {
     a.hs_pi[0] = (float)(kPi * 0.5 * a.h * kPi * f->p[0]);
     a.hs_pi[1] = (float)(kPi * a.h * kPi * f->p[0]);
+    const double hx = -kPi * a.h * kPi * f->p[0];
+    a.hx_pi[0] = (float)(0.5 * hx);
+    a.hx_pi[1] = (float)hx;
+    a.hx_pi[2] = (float)(hx / 6.0);
+    a.hx_pi_lo = (float)(hx / 6.0 - (double)a.hx_pi[2]);
+    a.hs_pi6 = (float)(kPi * a.h / 6.0 * kPi * f->p[0]);
+    a.hs_pi6_lo = (float)(kPi * a.h / 6.0 * kPi * f->p[0] - (double)a.hs_pi6);
   }
   const double hsc[3] = {0.5 * a.h, a.h, a.h / 6.0};
   for (int s = 0; s < 3; ++s)
@@ -290,6 +300,8 @@ AdvArgs make_adv_args(const ftle_mesh* m, const ftle_flow* f, double t0, double 
   double angle, diff;
   if (rotation_bounds(f, a.h, &angle, &diff)) a.rot_safe = rotation_unchecked(angle, diff) ? 1 : 0;
   a.carry_ok = carry_allowed(f, a.rot_safe != 0, angle);
+  // the double gyre's carried step drops th^5 / 120 of each step's turn: at most 2.8e-10 there
+  a.dg_carry = f->kind == FTLE_FLOW_DOUBLE_GYRE && a.rot_safe && angle <= (double)kCarryAngleMax * (1.0 - 1e-3);
   a.abc_refresh = a.carry_ok ? kAbcRefreshDefault : 1;
   return a;
 }
@@ -431,6 +443,8 @@ int run_advect(const ftle_mesh* m, const ftle_flow* fl, double t0, double T, dou
     if (rc) return rc;
     a.dg64 = 1;
   }
+  if (prec == P32C && a.dg_carry)
+    return launch_advect_dg_carry(m->coord_fp64 != 0, a, L.advect_shape ? L.advect_block : 0, L.advect_bps, s);
   int block = L.advect_block;
   if (prec == P64 && block > 128) block = 128;
   // by default a grid of 8192 / block blocks per SM (32 of 256 threads), more than fit at once:

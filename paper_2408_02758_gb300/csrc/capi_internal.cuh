@@ -24,6 +24,7 @@ struct Launch {
   double refine_kappa = 4e-4;
   int advect_block = 256;
   int advect_bps = 0;     // resident blocks per SM the advection grid is sized for (0: 2048/block)
+  bool advect_shape = false;  // advect_block set by the caller
   int grad_block = 256;
   int refine_lanes = 32;
   bool defer_fp64 = false;
@@ -63,6 +64,9 @@ int launch_advect_dg(int prec, int out, bool coord64, const AdvArgs& args, int g
                      size_t smem, cudaStream_t stream);
 int launch_advect_abc(int prec, int out, bool coord64, const AdvArgs& args, int grid, int block,
                       size_t smem, cudaStream_t stream);
+// Compensated double-gyre advection with carried sines and cosines (AdvArgs::dg_carry); block 0: the
+// launch shape of its own choice, blocks_per_sm 0: no limit on the grid.
+int launch_advect_dg_carry(bool coord64, const AdvArgs& args, int block, int blocks_per_sm, cudaStream_t s);
 // Double-precision advection of the double gyre's nodes in its domain, on the FP32 pipes.
 int launch_advect_dg64(bool coord64, const AdvArgs& args, cudaStream_t s);
 // Run-parallel float-float re-advection of a compensated 2D double-gyre flowmap (needs the run

@@ -268,13 +268,14 @@ struct FlowArgs {
 // residual, so that 2a + b is exactly 1 and the walls x = 0, 2 stay invariant in float
 // arithmetic.  sin(omega t) = sin(pi u), u = (omega/pi) t formed and reduced to [-1/2, 1/2] in
 // double, then evaluated by sinpif: the argument keeps double accuracy, the value float.
-// Returns (a, b_l); b_h = fmaf(-2, a, 1).
-__device__ __forceinline__ float2 dg_coef(double eps, double nu, double t0, double half_h, int m) {
+// Returns (a, b_l); b_h = fmaf(-2, a, 1).  eps_lo is what float(eps) leaves of eps: without it
+// (plain float) a's relative bias of up to 6e-8 acts on every node like a change of eps.
+__device__ __forceinline__ float2 dg_coef(double eps, float eps_lo, double nu, double t0, double half_h, int m) {
   double u = nu * (t0 + half_h * (double)m);
   double k = rint(u);
   float s = sinpif((float)(u - k));
   if (((long long)k) & 1) s = -s;  // sin(pi (k + r)) = (-1)^k sin(pi r)
-  float a = (float)eps * s;
+  float a = fmaf((float)eps, s, eps_lo * s);
   float bh, bl;
   two_sum(1.0f, -2.0f * a, bh, bl);
   return make_float2(a, bl);

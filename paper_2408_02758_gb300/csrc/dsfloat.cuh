@@ -159,6 +159,36 @@ __device__ __forceinline__ void ds_sincospi(dsf x, dsf& s, dsf& c) {
   ds_rotate(__ldg(reinterpret_cast<const float4*>(kDS_SINPI512_TAB) + (int)j + 512), su, cu, s, c);
 }
 
+// a + (b s + a cm) from a table entry's pair (a, b) and s = sin t, cm = cos t - 1 of a small angle
+// (|t| <= pi/1024): the small terms are summed first, then added to a once.
+__device__ __forceinline__ dsf ds_turn(float ah, float al, float bh, float bl, float sh, float sl, float cmh,
+                                         float cml) {
+  const float p = __fmul_rn(bh, sh);
+  const float pe = fmaf(bl, sh, fmaf(bh, sl, fmaf(bh, sh, -p)));
+  const float r = fmaf(ah, cmh, p);
+  const float re = fmaf(al, cmh, fmaf(ah, cml, fmaf(ah, cmh, __fsub_rn(p, r))));
+  const dsf v = ds_fast(ah, r);
+  return ds_make(v.h, __fadd_rn(v.l, __fadd_rn(al, __fadd_rn(re, pe))));
+}
+
+// (sin, cos)(pi x) of a float-float x, |x| < 2^12: as ds_sincospi (512 x = j + u, (sin, cos)(pi j/512)
+// from the table, the rest by Taylor) with the period folded into the table index, the integer held
+// in the low bits of the magic-rounded 512 x.  x.h - j/512 is exact.  Error 1.3e-15 rms, 1e-14 at most.
+__device__ __forceinline__ void ds_sincospi_fold(dsf x, dsf& s, dsf& c) {
+  const float m = fmaf(x.h, 512.0f, kRoundMagic);
+  const float j = __fsub_rn(m, kRoundMagic);
+  const float4 e = __ldg(reinterpret_cast<const float4*>(kDS_SINPI512_TAB) + ((__float_as_int(m) & 1023) ^ 512));
+  // normalized: where 512 x is near j the low part of x would otherwise round the angle at 2^-46
+  const dsf u = ds_fast(fmaf(j, -1.0f / 512.0f, x.h), x.l);
+  const dsf t = ds_mul_u(u, tc<1, true>());
+  const float t2 = t.h * t.h;
+  const dsf su = ds_fast(t.h, fmaf(t.h * t2, fmaf(t2, 1.0f / 120.0f, -1.0f / 6.0f), t.l));
+  const dsf tt = ds_mul_u(t, t);
+  const float cmh = -0.5f * tt.h, cml = fmaf(-0.5f, tt.l, tt.h * tt.h * (1.0f / 24.0f));
+  s = ds_turn(e.x, e.y, e.z, e.w, su.h, su.l, cmh, cml);
+  c = ds_turn(e.z, e.w, e.x, e.y, -su.h, -su.l, cmh, cml);
+}
+
 // sin(x), cos(x) of a float-float x: x = k pi/2 + r (the product in float-float), r = j/32 + u
 // (|u| <= 1/64, exact), (sin, cos)(j/32) from the table, u by the tiny series.
 __device__ __forceinline__ void ds_sincos(dsf x, dsf& s, dsf& c) {
