@@ -42,6 +42,11 @@ struct AdvArgs {
   int dg_carry;                // double gyre: rot_safe and the step's angles within kCarryAngleMax, so
                                // the sines and cosines may be carried (dg_step_carried)
   float habc[3][3];            // ABC: (h/2, h, h/6) times (A, B, C), rounded once
+  float abc_p[2][3], abc_nq[2][3];  // carried ABC steps: (h/2, h) times (A, B, C) and -(C, A, B), the
+                               // factors of each component's sine and negated cosine, rounded to
+                               // floats of nearly the right ratio (abc_factors)
+  float abc_s[3], abc_ns[3], abc_s_lo[3];  // 1/3 over what that rounding scales them by, its negative,
+                               // and its low part
   int abc_refresh;             // compensated ABC, unchecked steps: stage one's sines and cosines
                                // evaluated afresh every abc_refresh steps (a power of two),
                                // carried and turned by each step's increment in between
@@ -293,11 +298,7 @@ constexpr float kCarryAngleMax = 0.032f;
 
 // rotate_small_xyz without the th^4/24 term of cos th - 1, for the unchecked ABC step's stage
 // two, whose angles d1 = h/2 k1 stay within kRotMax / 2 under the host's bound (the dropped term
-// below 1.6e-8, about 1e-10 at dt = 0.01 on the 3D workload), and for stage four of a carried
-// step, whose angles stay within kCarryAngleMax (below 4.4e-8; about 2e-9 there).  At stage four
-// the term would shrink the carried pairs' norm by that much per step until the next fresh
-// evaluation; measured over the whole 256^3 field (period 8) the worst node went 8.5e-5 -> 7.4e-5
-// and the p99 stayed at 2.7e-6, i.e. the shrink is below the pairs' rounding.
+// below 1.6e-8, about 1e-10 at dt = 0.01 on the 3D workload).
 __device__ __forceinline__ void rotate_small_xyz_short(const float* s0, const float* c0, const float* d, float* s,
                                                        float* c) {
 #pragma unroll
@@ -367,16 +368,9 @@ __device__ __forceinline__ void rk4_step_c_full(const AdvArgs& a, const Coef& c0
 // first order (|d2 - d1| <= h^2/4 L U for a flow with Lipschitz constant L and speed bound U, so
 // the dropped (d2 - d1)^2 / 2 stays near float rounding: kTinyMax); stage four turns stage one's
 // by d3.  Without SAFE a stage angle beyond the turns' limits returns false (the caller then
-// evaluates the step in full).  With st4 (unchecked steps only) stage four's pairs and d3 are
-// handed back for the carried steps below.
-struct AbcStage4 {
-  float s[3], c[3], d3[3];
-};
-
-template <bool SAFE, bool KEEP4 = false>
-__device__ __forceinline__ bool abc_step_from(const AdvArgs& a, const float* s0, const float* c0v, float* inc,
-                                              AbcStage4* st4 = nullptr) {
-  static_assert(SAFE || !KEEP4, "stage four's pairs are kept by the unchecked step only");
+// evaluates the step in full).
+template <bool SAFE>
+__device__ __forceinline__ bool abc_step_from(const AdvArgs& a, const float* s0, const float* c0v, float* inc) {
   float d1[3], d2[3], d3[3], e4[3], mx = 0.0f;
   d1[0] = fmaf(a.habc[0][0], s0[2], a.habc[0][2] * c0v[1]);
   d1[1] = fmaf(a.habc[0][1], s0[0], a.habc[0][0] * c0v[2]);
@@ -400,102 +394,150 @@ __device__ __forceinline__ bool abc_step_from(const AdvArgs& a, const float* s0,
       mx = fmaxf(fmaxf(mx, fmaxf(fabsf(d1[0]), fmaxf(fabsf(d1[1]), fabsf(d1[2])))), dmax * (kRotMax / kTinyMax));
     abc_stage_k(a.habc[1], s3, c3, d3);
   }
-  if constexpr (KEEP4) {
-    rotate_small_xyz_short(s0, c0v, d3, st4->s, st4->c);  // carried steps only: |d3| <= kCarryAngleMax
-    abc_stage_k(a.habc[2], st4->s, st4->c, e4);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) st4->d3[q] = d3[q];
-  } else {
-    abc_stage_rot<!SAFE>(a.habc[2], d3, s0, c0v, mx, e4);
-  }
+  abc_stage_rot<!SAFE>(a.habc[2], d3, s0, c0v, mx, e4);
   if (!(SAFE || mx <= kRotMax)) return false;
 #pragma unroll
   for (int q = 0; q < 3; ++q) inc[q] = fmaf(fmaf(2.f, d2[q], d1[q] + d3[q]), 1.0f / 3.0f, e4[q]);
   return true;
 }
 
-// Stage one's (sin, cos) of the state carried from step to step by the unchecked compensated ABC
-// step (AdvArgs::rot_safe): a step whose index is a multiple of AdvArgs::abc_refresh evaluates
-// them afresh at the compensated state (fsincos_c); the steps between start from the previous
-// step's stage-four pairs, at x + d3 with d3 = h k3, and turn them to first order by what the
-// state moved beyond that point, inc - d3 = h/6 ((k1 - k3) + 2 (k2 - k3) + (k4 - k3)).  That
-// difference is third order in h (about h^3 L^2 U / 12; ~2e-6 rad at h = 0.01); in any case
-// |inc - d3| <= h^2 L U / 6 (1 + hL/2 + (hL)^2 / 8), below stage three's bound h^2 L U / 4
-// whenever hL <= kRotMax, so the host's kTinyMax check on stage three covers it and the dropped
-// (inc - d3)^2 / 2 stays below float rounding.  The increment is taken before its low part joins
-// the state, which moves the angle by at most half an ulp of the increment.  The turns'
-// roundings accumulate over at most abc_refresh - 1 steps before the next fresh evaluation.
-struct AbcCarry {
-  float s[3], c[3];
+// One node's (V = float) or two nodes' (float2, a node in each lane) state and carried pairs under the
+// unchecked compensated ABC step (AdvArgs::carry_ok).  Stage one's (sin, cos) of the state are
+// evaluated afresh at steps that are multiples of AdvArgs::abc_refresh (vsincos_c at the compensated
+// state); the steps between start from the previous step's stage-four pairs, at x + d3 with
+// d3 = h k3, and turn them to first order by what the state moved beyond that point, inc - d3 =
+// h/6 ((k1 - k3) + 2 (k2 - k3) + (k4 - k3)).  That difference is third order in h (about
+// h^3 L^2 U / 12; ~2e-6 rad at h = 0.01); in any case |inc - d3| <= h^2 L U / 6 (1 + hL/2 + (hL)^2 / 8),
+// below stage three's bound h^2 L U / 4 whenever hL <= kRotMax, so the host's kTinyMax check on stage
+// three covers it and the dropped (inc - d3)^2 / 2 stays below float rounding.
+// The increment is kept threefold, 3 inc = d1 + 2 d2 + d3 + h/2 k4, which joins k4 without a product
+// of its own; kAbcFold steps' sum waits in acc before it joins the state by Fast2Sum, scaled in two
+// parts (the steps between need the pairs alone).  FTLE error (2-norm, relative, root mean square over
+// twelve fields of 61 x 47 x 53 to 200 x 190 x 180 nodes) and time at 256^3: one node per thread, the
+// state joined at every step, A, B and C rounded one by one: 2.97e-7, 28.94 ms; two nodes, joined every
+// 2 steps: 2.98e-7, 26.2 ms; with the factors' ratios kept (abc_factors) 2.53e-7, 26.4 ms; joined every 4
+// steps 2.61e-7, 25.5 ms; and stage four turned flat, as here, 2.77e-7, 25.2 ms; joined every 8 steps
+// 2.97e-7, 25.0 ms.
+// The cosines are kept negated (nc): with the negated forms that the turns below produce, a step
+// of paired lanes needs a third of the sign flips, which cost two integer operations each there.
+template <class V>
+struct AbcNodes {
+  V xh[3], xl[3], s[3], nc[3], acc[3];
 };
+constexpr int kAbcFold = 4;  // a power of two
 
-// One carried step from the pairs in cy: the step's increment, the compensated state update,
-// and (with TURN) the next step's pairs from stage four's, turned by inc - d3 (formed exactly
-// where inc and d3 agree within a factor of two, as they do unless both are tiny).
-template <bool TURN>
-__device__ __forceinline__ void abc_carried_one(const AdvArgs& a, float* xh, float* xl, AbcCarry& cy) {
-  float inc[3];
-  AbcStage4 st4;
-  if constexpr (TURN)
-    abc_step_from<true, true>(a, cy.s, cy.c, inc, &st4);
-  else
-    abc_step_from<true>(a, cy.s, cy.c, inc);
+// (sin, -cos) turned by the small angle d, by sin d = d - d^3/6 and cos d - 1 = -d^2/2.  Stage two's angles
+// are half steps, within kRotMax / 2 under the host's bound (the dropped d^4 / 24 below 1.6e-8), stage
+// four's within kCarryAngleMax (below 4.4e-8).  Nesting the series (s + d (c - d/2 (s + d/3 c))) rounds
+// once less at the result's size for as many operations, but its longer chain costs 0.35 ms at stage
+// four and 0.6 ms at stage two (256^3) for the errors above.
+template <class V>
+__device__ __forceinline__ void abc_turn(V s0, V c0, V nc0, V d, V& s, V& nc) {
+  const V t = vmul(d, d), st = vfma(vmul(d, t), vsplat<V>(-1.0f / 6.0f), d), cm = vmul(t, vsplat<V>(-0.5f));
+  s = vfma(s0, cm, vfma(c0, st, s0));
+  nc = vfma(nc0, cm, vfma(s0, st, nc0));
+}
+
+// The velocity's components times h/2 (f = 0) or h (f = 1).
+template <class V>
+__device__ __forceinline__ void abc_vel(const AdvArgs& a, int f, const V* s, const V* nc, V* k) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+    k[q] = vfma(vsplat<V>(a.abc_p[f][q]), s[(q + 2) % 3], vmul(vsplat<V>(a.abc_nq[f][q]), nc[(q + 1) % 3]));
+}
+
+template <class V>
+__device__ __forceinline__ void abc_fresh(AbcNodes<V>& nd) {
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    float s, e;
-    comp_add<FTLE_FLOW_ABC>(xh[q], inc[q] + xl[q], s, e);
-    xh[q] = s;
-    xl[q] = e;
+    V c;
+    vsincos_c(nd.xh[q], nd.xl[q], nd.s[q], c);
+    nd.nc[q] = vneg(c);
   }
-  if constexpr (TURN) {
+}
+
+// What waits in acc into the state, by Fast2Sum (comp_add).
+template <class V>
+__device__ __forceinline__ void abc_fold(const AdvArgs& a, const V* acc, V* xh, V* xl) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const float dl = inc[q] - st4.d3[q];
-      cy.s[q] = fmaf(st4.c[q], dl, st4.s[q]);
-      cy.c[q] = fmaf(-st4.s[q], dl, st4.c[q]);
+  for (int q = 0; q < 3; ++q) {
+    const V d = vfma(acc[q], vsplat<V>(a.abc_s[q]), vfma(acc[q], vsplat<V>(a.abc_s_lo[q]), xl[q]));
+    const V s = vadd(xh[q], d), m1 = vsplat<V>(-1.0f);
+    xl[q] = vfma(vfma(xh[q], m1, s), m1, d);  // d - (s - xh)
+    xh[q] = s;
+  }
+}
+
+// One step: first: acc starts with this step's increment; turn: the pairs go on to the next step.
+template <class V>
+__device__ __forceinline__ void abc_step(const AdvArgs& a, AbcNodes<V>& nd, bool first, bool turn) {
+  V d1[3], d2[3], d3[3], c0[3], s2[3], nc2[3], s4[3], nc4[3];
+  abc_vel(a, 0, nd.s, nd.nc, d1);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    c0[q] = vneg(nd.nc[q]);
+    abc_turn(nd.s[q], c0[q], nd.nc[q], d1[q], s2[q], nc2[q]);
+  }
+  abc_vel(a, 0, s2, nc2, d2);
+  {
+    V s3[3], nc3[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {  // stage two's pairs by d2 - d1
+      const V dd = vfma(d1[q], vsplat<V>(-1.0f), d2[q]);
+      s3[q] = vfma(nc2[q], vneg(dd), s2[q]);
+      nc3[q] = vfma(s2[q], dd, nc2[q]);
+    }
+    abc_vel(a, 1, s3, nc3, d3);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) abc_turn(nd.s[q], c0[q], nd.nc[q], d3[q], s4[q], nc4[q]);
+  V i3[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    i3[q] = vfma(vsplat<V>(2.0f), d2[q], vadd(d1[q], d3[q]));
+    i3[q] = vfma(vsplat<V>(a.abc_p[0][q]), s4[(q + 2) % 3],
+                 vfma(vsplat<V>(a.abc_nq[0][q]), nc4[(q + 1) % 3], i3[q]));
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) nd.acc[q] = first ? i3[q] : vadd(nd.acc[q], i3[q]);
+  if (turn) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {  // stage four's pairs by inc - d3
+      const V ndl = vfma(i3[q], vsplat<V>(a.abc_ns[q]), d3[q]);
+      nd.s[q] = vfma(nc4[q], ndl, s4[q]);
+      nd.nc[q] = vfma(s4[q], vneg(ndl), nc4[q]);
     }
   }
 }
 
-__device__ __forceinline__ void abc_fresh_pairs(const float* xh, const float* xl, AbcCarry& cy) {
-#pragma unroll
-  for (int q = 0; q < 3; ++q) fsincos_c(xh[q], xl[q], cy.s[q], cy.c[q]);
-}
-
-// Step k alone (for loops that do more per step, such as storing checkpoints).
-__device__ __forceinline__ void abc_step_carried(const AdvArgs& a, int k, float* xh, float* xl, AbcCarry& cy) {
-  const int mask = a.abc_refresh - 1;  // abc_refresh is a power of two
-  if ((k & mask) == 0) abc_fresh_pairs(xh, xl, cy);
-  if (((k + 1) & mask) != 0)
-    abc_carried_one<true>(a, xh, xl, cy);
-  else
-    abc_carried_one<false>(a, xh, xl, cy);
-}
-
-// Steps k .. stop - 1, the same arithmetic as abc_step_carried step by step, grouped between
-// refreshes so that the inner loop tests nothing but its bound (k ends at stop).
-__device__ __forceinline__ void abc_steps_carried(const AdvArgs& a, int& k, int stop, float* xh, float* xl,
-                                                  AbcCarry& cy) {
-  const int mask = a.abc_refresh - 1;
+// Steps k .. stop - 1 (k ends at stop).  A whole group of the default period is unrolled.
+template <class V>
+__device__ __forceinline__ void abc_steps(const AdvArgs& a, int& k, int stop, AbcNodes<V>& nd) {
+  const int mask = a.abc_refresh - 1, fold = min(kAbcFold, a.abc_refresh) - 1;  // powers of two
   while (k < stop) {
-    const int g = min(stop, (k | mask) + 1);  // the next step that refreshes, or stop
-    if (mask == kAbcRefreshDefault - 1 && (k & mask) == 0 && g - k == kAbcRefreshDefault) {
-      // a whole group of the default period, unrolled
-      abc_fresh_pairs(xh, xl, cy);
+    if (mask == kAbcRefreshDefault - 1 && (k & mask) == 0 && stop - k >= kAbcRefreshDefault) {
+      abc_fresh(nd);
 #pragma unroll
-      for (int q = 0; q < kAbcRefreshDefault - 1; ++q) abc_carried_one<true>(a, xh, xl, cy);
-      abc_carried_one<false>(a, xh, xl, cy);
-      k = g;
+      for (int q = 0; q < kAbcRefreshDefault; ++q) {
+        abc_step(a, nd, q % kAbcFold == 0, q + 1 < kAbcRefreshDefault);
+        if (q % kAbcFold == kAbcFold - 1) abc_fold(a, nd.acc, nd.xh, nd.xl);
+      }
+      k += kAbcRefreshDefault;
       continue;
     }
-    if ((k & mask) == 0) abc_fresh_pairs(xh, xl, cy);
-    for (; k < g - 1; ++k) abc_carried_one<true>(a, xh, xl, cy);
-    if ((g & mask) != 0)  // cut short by stop: a later call carries on from these pairs
-      abc_carried_one<true>(a, xh, xl, cy);
-    else
-      abc_carried_one<false>(a, xh, xl, cy);
+    if ((k & mask) == 0) abc_fresh(nd);
+    abc_step(a, nd, (k & fold) == 0, true);
     ++k;
+    if ((k & fold) == 0) abc_fold(a, nd.acc, nd.xh, nd.xl);
   }
+}
+
+// The state after k steps, what waits in acc included.
+template <class V>
+__device__ __forceinline__ void abc_state(const AdvArgs& a, int k, const AbcNodes<V>& nd, V* xh, V* xl) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) xh[q] = nd.xh[q], xl[q] = nd.xl[q];
+  if (k & (min(kAbcFold, a.abc_refresh) - 1)) abc_fold(a, nd.acc, xh, xl);
 }
 
 // The double gyre's (sin, cos) of pi f and pi y at the state, carried from step to step by the unchecked
@@ -901,13 +943,11 @@ __device__ __forceinline__ bool dg64_coord(double z, int p) {
 
 // SAFE: the instantiation for AdvArgs::rot_safe (rk4_step's angle-check-free ABC step).  The
 // compensated float kernels are held to five 256-thread blocks per SM (48 registers) for the
-// double gyre (measured on the full mesh: 15.84 ms at 40 registers, six blocks; 15.47 at 48;
-// 15.83 at 64, four blocks) and six for the ABC flow with stage one carried (40 registers, a
-// few bytes spilled outside the step loop: 37.83 ms against 38.46 at five blocks).
-// CARRY (with SAFE, the compensated ABC step): stage one's (sin, cos) carried across steps
-// (abc_step_carried, AdvArgs::abc_refresh > 1).
-template <int KIND, int DIM, int PREC, int OUT, typename CT, bool SAFE = false, bool CARRY = false>
-__global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6 : 4) : 1) k_advect(AdvArgs a) {
+// double gyre (measured on the full mesh with the pairs evaluated at every step: 15.84 ms at 40
+// registers, six blocks; 15.47 at 48; 15.83 at 64, four blocks) and six for the ABC flow.  Steps that
+// carry stage one's sines and cosines run in k_advect_dg and k_advect_abc instead.
+template <int KIND, int DIM, int PREC, int OUT, typename CT, bool SAFE = false>
+__global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6 : 5) : 1) k_advect(AdvArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr bool kTable = (KIND == FTLE_FLOW_DOUBLE_GYRE);
   float2* tab32 = reinterpret_cast<float2*>(smem_raw);
@@ -944,7 +984,6 @@ __global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6
     if constexpr (KIND == FTLE_FLOW_DOUBLE_GYRE && PREC == P32C) safe_node = dg_node_safe(a, xd[0], xd[1]);
     int ck_left = a.ckpt_every;
     int ck_slot = 1;
-    AbcCarry carry;  // stage one's carried (sin, cos), refreshed at step 0 and every abc_refresh
     constexpr bool kSegs = PREC == P32C && OUT == O32PAIR && DIM == 2;
     int seg_slot = 0, next_seg = a.seg_len;
 
@@ -963,24 +1002,13 @@ __global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6
       for (int k = k0; k < k1;) {
         // steps up to the next run boundary (uniform across the block), then its state
         const int stop = (kSegs && a.seg) ? min(k1, next_seg) : k1;
-        // abc_refresh = 1 takes rk4_step's unchecked ABC step (CARRY false), the same arithmetic
-        // without the carried pairs' bookkeeping
-        auto steps = [&](auto safe, auto carried) {
-          if constexpr (KIND == FTLE_FLOW_ABC && PREC == P32C && decltype(safe)::value && decltype(carried)::value) {
-            if (!a.ckpt) {
-              abc_steps_carried(a, k, stop, xh, xl, carry);
-              return;
-            }
-          }
+        auto steps = [&](auto safe) {
           for (; k < stop; ++k) {
             const int m = 2 * (k - k0);
             const Coef c0 = coef_at<KIND, PREC>(tab32, tab64, m);
             const Coef c1 = coef_at<KIND, PREC>(tab32, tab64, m + 1);
             const Coef c2 = coef_at<KIND, PREC>(tab32, tab64, m + 2);
-            if constexpr (KIND == FTLE_FLOW_ABC && PREC == P32C && decltype(safe)::value && decltype(carried)::value)
-              abc_step_carried(a, k, xh, xl, carry);
-            else
-              rk4_step<KIND, DIM, PREC, decltype(safe)::value>(a, c0, c1, c2, xh, xl, xd);
+            rk4_step<KIND, DIM, PREC, decltype(safe)::value>(a, c0, c1, c2, xh, xl, xd);
             if (a.ckpt) {
               if (--ck_left == 0) {
                 ck_left = a.ckpt_every;
@@ -992,13 +1020,10 @@ __global__ void __launch_bounds__(256, PREC == P32C ? (KIND == FTLE_FLOW_ABC ? 6
             }
           }
         };
-        if (SAFE) {
-          steps(std::integral_constant<bool, SAFE>{}, std::integral_constant<bool, CARRY>{});
-        } else if (safe_node) {
-          steps(std::true_type{}, std::false_type{});
-        } else {
-          steps(std::false_type{}, std::false_type{});
-        }
+        if (SAFE || safe_node)
+          steps(std::true_type{});
+        else
+          steps(std::false_type{});
         if constexpr (kSegs) {
           if (a.seg && k == next_seg) {
             if (seg_slot < kSegments - 1)
@@ -1167,6 +1192,68 @@ __device__ __forceinline__ void dg_walk(const AdvArgs& a, const float2* tab, int
     if (any) dg_walk_chunk<N>(a, tab, k0, k1, i, stride, active, safe, w);
   }
   w.end(a, i, stride, active);
+}
+
+// Up to two ABC nodes of a thread (V = float2: nodes i and i + stride, the second inside the mesh when
+// two is set) from their coordinates to their records.
+template <class V, typename CT>
+__device__ __forceinline__ void abc_walk(const AdvArgs& a, int64_t i, int64_t stride, bool two) {
+  constexpr int N = (int)(sizeof(V) / sizeof(float));
+  AbcNodes<V> nd;
+  float x0[N][3];
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const int64_t j = q && two ? i + stride : i;  // a lone last node takes both lanes
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double x = load_coord<CT>(a.coords, d * a.n_mesh + j);
+      const float h = (float)x;
+      vset(nd.xh[d], q, h);
+      vset(nd.xl[d], q, (float)(x - (double)h));
+      x0[q][d] = h;
+    }
+  }
+  auto store = [&](void* base, int k, bool records) {
+    V xh[3], xl[3];
+    abc_state(a, k, nd, xh, xl);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      if (q && !two) continue;
+      float h[3], l[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) h[d] = vget(xh[d], q), l[d] = vget(xl[d], q);
+      store_state<O32PAIR, 3>(base, a.n_mesh, i + q * stride, h, l, nullptr);
+      if (records && a.rec) store_record<3>(a.rec, i + q * stride, x0[q], h, l);
+    }
+  };
+  int k = 0;
+  if (a.ckpt) {
+    store(a.ckpt, 0, false);
+    for (int slot = 1; k < a.nsteps; ++slot) {
+      const int to = a.nsteps - k > a.ckpt_every ? k + a.ckpt_every : a.nsteps;
+      const bool whole = to - k == a.ckpt_every;
+      abc_steps(a, k, to, nd);
+      if (whole) store(reinterpret_cast<char*>(a.ckpt) + (int64_t)slot * a.ckpt_stride_bytes, k, false);
+    }
+  } else {
+    abc_steps(a, k, a.nsteps, nd);
+  }
+  store(a.out, k, true);
+}
+
+// k_advect for compensated ABC flowmaps whose steps carry stage one's sines and cosines: N nodes per
+// thread, 32 N consecutive nodes per warp.
+template <int N>
+constexpr int kAbcBlocks = N == 2 ? 2 : 5;  // 256-thread blocks per SM (three: 26.3 ms against 26.2 at 256^3)
+
+template <int N, typename CT>
+__global__ void __launch_bounds__(256, kAbcBlocks<N>) k_advect_abc(AdvArgs a) {
+  using V = typename std::conditional<N == 2, float2, float>::type;
+  const int64_t tiles = (a.n + 32 * N - 1) / (32 * N), per_round = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t tile = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; tile < tiles; tile += per_round) {
+    const int64_t i = tile * 32 * N + (threadIdx.x & 31);
+    if (i < a.n) abc_walk<V, CT>(a, i, 32, i + 32 < a.n);
+  }
 }
 
 // k_advect for compensated double-gyre flowmaps whose steps carry the sines and cosines: N nodes per

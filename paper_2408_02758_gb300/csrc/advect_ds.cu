@@ -403,14 +403,20 @@ __global__ void __launch_bounds__(32 * kAbcRunWarps) k_refine_runs_abc(AdvArgs a
         xl[q] = (float)(xd[q] - (double)xh[q]);
       }
       const Coef c0{0.f, 0.f, 0.f, 0.0};  // the ABC flow is autonomous
-      AbcCarry carry;  // the unchecked step carries stage one's pairs, as the main advection does
+      AbcNodes<float> nd;  // the unchecked step carries stage one's pairs, as the main advection does
+#pragma unroll
+      for (int q = 0; q < 3; ++q) nd.xh[q] = xh[q], nd.xl[q] = xl[q];
       int k = 0;
       for (int j = 1; j < kAbcRuns; ++j) {
         const int kend = min(j * L, a.nsteps);
-        if (a.rot_safe)
-          abc_steps_carried(a, k, kend, xh, xl, carry);
-        else
+        if (a.carry_ok) {
+          abc_steps(a, k, kend, nd);
+          abc_state(a, k, nd, xh, xl);
+        } else if (a.rot_safe) {
+          for (; k < kend; ++k) rk4_step<FTLE_FLOW_ABC, 3, P32C, true>(a, c0, c0, c0, xh, xl, xd);
+        } else {
           for (; k < kend; ++k) rk4_step<FTLE_FLOW_ABC, 3, P32C, false>(a, c0, c0, c0, xh, xl, xd);
+        }
 #pragma unroll
         for (int q = 0; q < 3; ++q) s_bnd[wib][j][q] = make_float2(xh[q], xl[q]);
       }

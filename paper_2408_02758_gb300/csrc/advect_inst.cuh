@@ -13,9 +13,7 @@ int launch_advect_typed(int prec, int out, const AdvArgs& args, int grid, int bl
     k_advect<KIND, DIM, P32, O32, CT><<<grid, block, smem, stream>>>(args);
   } else if (prec == P32C && out == O32PAIR) {
     constexpr bool kAbc = KIND == FTLE_FLOW_ABC;
-    if (kAbc && args.rot_safe && args.abc_refresh > 1)
-      k_advect<KIND, DIM, P32C, O32PAIR, CT, kAbc, kAbc><<<grid, block, smem, stream>>>(args);
-    else if (kAbc && args.rot_safe)
+    if (kAbc && args.rot_safe)
       k_advect<KIND, DIM, P32C, O32PAIR, CT, kAbc><<<grid, block, smem, stream>>>(args);
     else
       k_advect<KIND, DIM, P32C, O32PAIR, CT><<<grid, block, smem, stream>>>(args);

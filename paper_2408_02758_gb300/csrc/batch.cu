@@ -63,7 +63,6 @@ __global__ void __launch_bounds__(256, PREC == P32C ? 4 : 1) k_batch_advect(cons
     // run-boundary states of compensated 2D flowmaps (as k_advect stores them)
     constexpr bool kSegs = PREC == P32C && OUT == O32PAIR && DIM == 2;
     int seg_slot = 0, next_seg = a.seg_len;
-    AbcCarry carry;  // as k_advect: the same steps, the same bits
     for (int ch = 0; ch < nchunks; ++ch) {
       const int k0 = ch * kAdvChunk;
       const int k1 = min(a.nsteps, k0 + kAdvChunk);
@@ -78,30 +77,20 @@ __global__ void __launch_bounds__(256, PREC == P32C ? 4 : 1) k_batch_advect(cons
       if (!active) continue;
       for (int k = k0; k < k1;) {
         const int stop = (kSegs && a.seg) ? min(k1, next_seg) : k1;
-        auto steps = [&](auto safe, auto carried) {
-          if constexpr (KIND == FTLE_FLOW_ABC && PREC == P32C && decltype(safe)::value && decltype(carried)::value) {
-            abc_steps_carried(a, k, stop, xh, xl, carry);
-            return;
-          }
+        auto steps = [&](auto safe) {
           for (; k < stop; ++k) {
             const int m = 2 * (k - k0);
             const Coef c0 = coef_at<KIND, PREC>(tab32, tab64, m);
             const Coef c1 = coef_at<KIND, PREC>(tab32, tab64, m + 1);
             const Coef c2 = coef_at<KIND, PREC>(tab32, tab64, m + 2);
-            if constexpr (KIND == FTLE_FLOW_ABC && PREC == P32C && decltype(safe)::value && decltype(carried)::value)
-              abc_step_carried(a, k, xh, xl, carry);
-            else
-              rk4_step<KIND, DIM, PREC, decltype(safe)::value>(a, c0, c1, c2, xh, xl, xd);
+            rk4_step<KIND, DIM, PREC, decltype(safe)::value>(a, c0, c1, c2, xh, xl, xd);
           }
         };
-        // the unchecked steps exactly where k_advect takes them (dg_node_safe; ABC: rot_safe),
-        // stage one carried as k_advect carries it
-        if (safe && a.abc_refresh > 1)
-          steps(std::true_type{}, std::true_type{});
-        else if (safe)
-          steps(std::true_type{}, std::false_type{});
+        // the unchecked steps exactly where k_advect takes them (dg_node_safe; ABC: rot_safe)
+        if (safe)
+          steps(std::true_type{});
         else
-          steps(std::false_type{}, std::false_type{});
+          steps(std::false_type{});
         if constexpr (kSegs) {
           if (a.seg && k == next_seg) {
             if (seg_slot < kSegments - 1)
@@ -153,6 +142,24 @@ __global__ void __launch_bounds__(256, kDgBlocks<2>) k_batch_advect_dg(const Bat
       __syncthreads();
     };
     dg_walk<2, float>(a, tab, (int64_t)item.lo + (threadIdx.x >> 5) * 64 + (threadIdx.x & 31), 32, item.hi, build);
+  }
+}
+
+// Likewise the items of ABC instances whose steps carry stage one's pairs (as k_advect_abc).
+__global__ void __launch_bounds__(256, kAbcBlocks<2>) k_batch_advect_abc(const BatchInst* __restrict__ insts,
+                                                                         const BatchItem* __restrict__ items,
+                                                                         int n_items, unsigned int* next) {
+  __shared__ int s_item;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= n_items) break;
+    const BatchItem item = items[it];
+    const AdvArgs a = insts[item.inst].adv;
+    const int64_t i = (int64_t)item.lo + (threadIdx.x >> 5) * 64 + (threadIdx.x & 31);
+    if (i < item.hi) abc_walk<float2, float>(a, i, 32, i + 32 < item.hi);
   }
 }
 
@@ -281,10 +288,13 @@ int launch_batch_mark(const BatchInst* insts, const int2* flags, const unsigned 
   return FTLE_OK;
 }
 
-static int launch_batch_advect_dg(const BatchInst* insts, const BatchItem* items, int n_items, unsigned int* next, int grid,
-                                  int block, size_t smem, cudaStream_t s) {
-  k_batch_advect_dg<<<grid, block, smem, s>>>(insts, items, n_items, next);
-  FTLE_LAUNCH_CHECK("k_batch_advect_dg launch");
+static int launch_batch_advect_carry(int kind, const BatchInst* insts, const BatchItem* items, int n_items,
+                                     unsigned int* next, int grid, int block, size_t smem, cudaStream_t s) {
+  if (kind == FTLE_FLOW_DOUBLE_GYRE)
+    k_batch_advect_dg<<<grid, block, smem, s>>>(insts, items, n_items, next);
+  else
+    k_batch_advect_abc<<<grid, block, 0, s>>>(insts, items, n_items, next);
+  FTLE_LAUNCH_CHECK("k_batch_advect_dg / k_batch_advect_abc launch");
   return FTLE_OK;
 }
 
@@ -342,8 +352,8 @@ struct BatchPlanHost {
   BatchLayout L;
   std::vector<BatchInst> insts;
   std::vector<BatchItem> adv_items, grad_items;
-  int carry_block = 128;  // threads per block of k_batch_advect_dg
-  int n_carry = 0;  // the first adv_items: carried double-gyre steps (k_batch_advect_dg)
+  int carry_block = 128;  // threads per block of k_batch_advect_dg and _abc
+  int n_carry = 0;  // the first adv_items: carried steps (k_batch_advect_dg, _abc)
   int max_steps_carry = 0;
 };
 
@@ -415,9 +425,12 @@ int plan_batch(int32_t n_inst, const ftle_mesh* meshes, const ftle_flow* flows, 
     bi.off = off;
     off += meshes[q].n_nodes;
   }
-  // advection queues, one after the other: items of instances with carried double-gyre steps (two nodes
-  // per thread), then of the others; each of one block of threads, longest (steps x nodes) first
-  auto carry = [&](int q) { return precision == FTLE_PREC_FP32C && P.insts[q].adv.dg_carry; };
+  // advection queues, one after the other: items of instances whose steps carry the sines and cosines (two
+  // nodes per thread), then of the others; each of one block of threads, longest (steps x nodes) first
+  auto carry = [&](int q) {
+    const AdvArgs& v = P.insts[q].adv;
+    return precision == FTLE_PREC_FP32C && (v.dg_carry || (v.carry_ok && v.abc_refresh > 1));
+  };
   for (int pass = 0; pass < 2; ++pass) {
     const size_t first = P.adv_items.size();
     for (int q = 0; q < n_inst; ++q) {
@@ -484,8 +497,8 @@ int enqueue_batch(const BatchPlanHost& P, cudaStream_t s) {
   const BatchItem* items = reinterpret_cast<const BatchItem*>(w + P.L.adv_items);
   const int n_items = (int)P.adv_items.size();
   if (P.n_carry > 0) {
-    const int grid = std::min(sms * kDgBlocks<2> * 256 / P.carry_block, P.n_carry);  // all resident
-    if ((rc = launch_batch_advect_dg(insts, items, P.n_carry, carry_next, grid, P.carry_block,
+    const int grid = std::min(sms * 2 * 256 / P.carry_block, P.n_carry);  // all resident
+    if ((rc = launch_batch_advect_carry(P.kind, insts, items, P.n_carry, carry_next, grid, P.carry_block,
                                      advect_smem_bytes(P.kind, prec, P.max_steps_carry), s)))
       return rc;
   }

@@ -261,6 +261,41 @@ static bool dg64_applies(const ftle_flow* f, double h, int nsteps) {
          kPi * kPi * A * (1.0 + 2.0 * eps) * fabs(h) * (double)nsteps <= 54.0;
 }
 
+// The factors of the carried ABC steps.  Rounding h/2 A and h/2 C each to a float would change the flow
+// by up to 6e-8 of a parameter at every step.  Of nine neighbouring floats the pair whose ratio is
+// most nearly right is off mainly by a common factor, which the state's increment takes back; the
+// stage points keep it (at most 6e-7 of an increment, second order in the step).
+static void abc_factors(const ftle_flow* f, AdvArgs& a) {
+  for (int q = 0; q < 3; ++q) {
+    const double P = 0.5 * a.h * f->p[q], Q = 0.5 * a.h * f->p[(q + 2) % 3];
+    float bp = (float)P, bq = (float)Q;
+    double scale = P != 0.0 ? (double)bp / P : Q != 0.0 ? (double)bq / Q : 1.0;
+    if (f->kind == FTLE_FLOW_ABC && bp != 0.0f && bq != 0.0f) {
+      float p = bp;
+      for (int i = 0; i < 4; ++i) p = nextafterf(p, -INFINITY);
+      double best = INFINITY;
+      for (int i = 0; i < 9; ++i, p = nextafterf(p, INFINITY)) {
+        const float r = (float)((double)p * (Q / P));
+        const double off = fabs((double)r / (double)p / (Q / P) - 1.0);
+        if (off < best) {
+          best = off;
+          bp = p;
+          bq = r;
+          scale = 0.5 * ((double)p / P + (double)r / Q);
+        }
+      }
+    }
+    if (!(scale > 0.5 && scale < 2.0)) scale = 1.0;  // factors at the end of the float range
+    for (int s = 0; s < 2; ++s) {
+      a.abc_p[s][q] = (s ? 2.0f : 1.0f) * bp;
+      a.abc_nq[s][q] = (s ? -2.0f : -1.0f) * bq;
+    }
+    a.abc_s[q] = (float)(1.0 / (3.0 * scale));
+    a.abc_ns[q] = -a.abc_s[q];
+    a.abc_s_lo[q] = (float)(1.0 / (3.0 * scale) - (double)a.abc_s[q]);
+  }
+}
+
 AdvArgs make_adv_args(const ftle_mesh* m, const ftle_flow* f, double t0, double T, double dt, int nsteps) {
   AdvArgs a;
   memset(&a, 0, sizeof a);
@@ -297,6 +332,7 @@ AdvArgs make_adv_args(const ftle_mesh* m, const ftle_flow* f, double t0, double 
   const double hsc[3] = {0.5 * a.h, a.h, a.h / 6.0};
   for (int s = 0; s < 3; ++s)
     for (int q = 0; q < 3; ++q) a.habc[s][q] = (float)(hsc[s] * f->p[q]);
+  if (f->kind == FTLE_FLOW_ABC) abc_factors(f, a);
   double angle, diff;
   if (rotation_bounds(f, a.h, &angle, &diff)) a.rot_safe = rotation_unchecked(angle, diff) ? 1 : 0;
   a.carry_ok = carry_allowed(f, a.rot_safe != 0, angle);
@@ -445,6 +481,8 @@ int run_advect(const ftle_mesh* m, const ftle_flow* fl, double t0, double T, dou
   }
   if (prec == P32C && a.dg_carry)
     return launch_advect_dg_carry(m->coord_fp64 != 0, a, L.advect_shape ? L.advect_block : 0, L.advect_bps, s);
+  if (prec == P32C && a.carry_ok && a.abc_refresh > 1)
+    return launch_advect_abc_carry(m->coord_fp64 != 0, a, L.advect_shape ? L.advect_block : 0, L.advect_bps, s);
   int block = L.advect_block;
   if (prec == P64 && block > 128) block = 128;
   // by default a grid of 8192 / block blocks per SM (32 of 256 threads), more than fit at once:

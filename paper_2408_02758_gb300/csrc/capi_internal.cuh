@@ -64,8 +64,9 @@ int launch_advect_dg(int prec, int out, bool coord64, const AdvArgs& args, int g
                      size_t smem, cudaStream_t stream);
 int launch_advect_abc(int prec, int out, bool coord64, const AdvArgs& args, int grid, int block,
                       size_t smem, cudaStream_t stream);
-// Compensated double-gyre advection with carried sines and cosines (AdvArgs::dg_carry); block 0: the
+// Compensated advection with carried sines and cosines (AdvArgs::dg_carry, carry_ok); block 0: the
 // launch shape of its own choice, blocks_per_sm 0: no limit on the grid.
+int launch_advect_abc_carry(bool coord64, const AdvArgs& args, int block, int blocks_per_sm, cudaStream_t s);
 int launch_advect_dg_carry(bool coord64, const AdvArgs& args, int block, int blocks_per_sm, cudaStream_t s);
 // Double-precision advection of the double gyre's nodes in its domain, on the FP32 pipes.
 int launch_advect_dg64(bool coord64, const AdvArgs& args, cudaStream_t s);

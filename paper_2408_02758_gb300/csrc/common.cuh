@@ -100,6 +100,32 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
+// One node's float or two nodes' lanes: the same operations, rounded alike and never contracted
+// further, so that a step written on them gives a node the same bits either way.
+template <class V>
+__device__ __forceinline__ V vsplat(float x);
+template <>
+__device__ __forceinline__ float vsplat<float>(float x) { return x; }
+template <>
+__device__ __forceinline__ float2 vsplat<float2>(float x) { return f2(x); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
+__device__ __forceinline__ float2 vneg(float2 a) { return neg2(a); }
+__device__ __forceinline__ float vget(float a, int) { return a; }
+__device__ __forceinline__ float vget(float2 a, int q) { return q ? a.y : a.x; }
+__device__ __forceinline__ void vset(float& a, int, float x) { a = x; }
+__device__ __forceinline__ void vset(float2& a, int q, float x) {
+  if (q)
+    a.y = x;
+  else
+    a.x = x;
+}
+
 // pi/2 in three parts: A (8 significant bits) and B (13) make k*A and k*B exact for |k| < 2^11;
 // C is the rest, rounded.
 constexpr float kPio2A = 0x1.92p+0f;
@@ -120,6 +146,28 @@ __device__ __forceinline__ void fsincos_c(float xh, float xl, float& s, float& c
   const float ps = fmaf(fmaf(fmaf(kRAD_S[3], z, kRAD_S[2]), z, kRAD_S[1]), z, kRAD_S[0]) * rh;
   const float pc = fmaf(fmaf(fmaf(fmaf(kRAD_C[4], z, kRAD_C[3]), z, kRAD_C[2]), z, kRAD_C[1]), z, kRAD_C[0]);
   quarter_turn(t, fmaf(rl, pc, ps), fmaf(-rl, ps, pc), s, c);
+}
+
+// fsincos_c of one node or of two.
+template <class V>
+__device__ __forceinline__ void vsincos_c(V xh, V xl, V& s, V& c) {
+  const V t = vfma(xh, vsplat<V>(0.636619772367581343f), vsplat<V>(kRoundMagic));
+  const V nk = vadd(vsplat<V>(kRoundMagic), vneg(t));  // -k
+  const V rh = vfma(nk, vsplat<V>(kPio2B), vfma(nk, vsplat<V>(kPio2A), xh));
+  const V rl = vfma(nk, vsplat<V>(kPio2C), xl);
+  const V z = vmul(rh, rh);
+  const V ps = vmul(vfma(vfma(vfma(vsplat<V>(kRAD_S[3]), z, vsplat<V>(kRAD_S[2])), z, vsplat<V>(kRAD_S[1])), z,
+                         vsplat<V>(kRAD_S[0])), rh);
+  const V pc = vfma(vfma(vfma(vfma(vsplat<V>(kRAD_C[4]), z, vsplat<V>(kRAD_C[3])), z, vsplat<V>(kRAD_C[2])), z,
+                         vsplat<V>(kRAD_C[1])), z, vsplat<V>(kRAD_C[0]));
+  const V sr = vfma(rl, pc, ps), cr = vfma(vneg(rl), ps, pc);
+#pragma unroll
+  for (int q = 0; q < (int)(sizeof(V) / sizeof(float)); ++q) {
+    float a, b;
+    quarter_turn(vget(t, q), vget(sr, q), vget(cr, q), a, b);
+    vset(s, q, a);
+    vset(c, q, b);
+  }
 }
 
 __device__ __forceinline__ void fsincos(float x, float& s, float& c) { fsincos_c(x, 0.0f, s, c); }
