@@ -11,13 +11,11 @@
 // the FTLE of the first, relative: 4.5e-14 -> 9e-15.  18.35 -> 1.38 ms: 553 warp instructions per
 // lane-step, the FP32 pipe 59 % busy, held by the 3.4 warps that each SM sub-partition has at this size.
 //
-// Two lanes per node, as in the float-float re-advection: lane 0 carries x and evaluates
-// (sin, cos)(pi f), lane 1 carries y and evaluates (sin, cos)(pi y); the argument is
-// f = z + a_p z (z - 2) on both, with a_1 = 0.
+// Two lanes per node, as in the float-float re-advection (dg_pair_vel).
 #include <math.h>
 
 #include "capi_internal.cuh"
-#include "dsfloat.cuh"
+#include "dg_pair.cuh"
 
 namespace ftle {
 
@@ -25,24 +23,10 @@ constexpr int kDg64Chunk = 1024;  // steps per coefficient table (16 bytes a hal
 constexpr int kDg64Warps = 8;     // warps per block, at most
 constexpr int kDg64Blocks = 4;    // blocks per SM: 32 warps of 64 registers
 
-// This lane's velocity component at z without its factor (-pi A, pi A), with the half step's
-// coefficients (a, b = 1 - 2a): sin(pi f) cos(pi y) on lane 0, sin(pi y) cos(pi f) f_x on lane 1.
-__device__ __forceinline__ dsf dg64_vel(int p, const dsf& z, const float4& ab) {
-  const dsf t1 = ds_mul_u(ds_make(p ? 0.f : ab.x, p ? 0.f : ab.y), z);
-  dsf z2 = ds_fast(-2.0f, z.h);  // z - 2, normalized for the nodes near the wall at 2
-  z2 = ds_fast(z2.h, __fadd_rn(z2.l, z.l));
-  const dsf f = ds_add_u(z, ds_mul_u(t1, z2));
-  const dsf fx = ds_add_u(ds_make(2.0f * t1.h, 2.0f * t1.l), ds_make(ab.z, ab.w));
-  const float gh = __shfl_xor_sync(0xffffffffu, fx.h, 1), gl = __shfl_xor_sync(0xffffffffu, fx.l, 1);
-  dsf sn, cs;
-  ds_sincospi_fold(f, sn, cs);
-  const dsf cq = ds_make(__shfl_xor_sync(0xffffffffu, cs.h, 1), __shfl_xor_sync(0xffffffffu, cs.l, 1));
-  return ds_mul_u(ds_mul_u(sn, cq), ds_make(p ? gh : 1.0f, p ? gl : 0.0f));
-}
-
 template <typename CT>
 __global__ void __launch_bounds__(32 * kDg64Warps, kDg64Blocks) k_advect_dg64(AdvArgs a) {
   __shared__ float4 s_ab[2 * kDg64Chunk + 1];
+  constexpr unsigned int kFull = 0xffffffffu;
   const int p = threadIdx.x & 1, lane = threadIdx.x & 31;
   const double scale = (p ? kPi : -kPi) * a.p[0];
   const dsf S2 = ds_from_double(0.5 * a.h * scale), S1 = ds_from_double(a.h * scale);
@@ -75,7 +59,7 @@ __global__ void __launch_bounds__(32 * kDg64Warps, kDg64Blocks) k_advect_dg64(Ad
         __syncthreads();
         for (int m = threadIdx.x; m <= 2 * (k1 - k0); m += blockDim.x) {
           const dsf c = ds_from_double(a.p[1] * sin(a.p[2] * (a.t0 + 0.5 * a.h * (double)(2 * k0 + m))));
-          const dsf b = ds_add_f(ds_make(-2.0f * c.h, -2.0f * c.l), 1.0f);
+          const dsf b = dg_pair_b(c);
           s_ab[m] = make_float4(c.h, c.l, b.h, b.l);
         }
         __syncthreads();
@@ -85,11 +69,11 @@ __global__ void __launch_bounds__(32 * kDg64Warps, kDg64Blocks) k_advect_dg64(Ad
       float4 c0 = s_ab[0];
       for (int k = k0; k < k1; ++k) {
         const float4 c1 = s_ab[2 * (k - k0) + 1], c2 = s_ab[2 * (k - k0) + 2];
-        const dsf x = ds_make(xh, xm);
-        const dsf w1 = dg64_vel(p, x, c0);
-        const dsf w2 = dg64_vel(p, ds_add_u(x, ds_mul_u(S2, w1)), c1);
-        const dsf w3 = dg64_vel(p, ds_add_u(x, ds_mul_u(S2, w2)), c1);
-        const dsf w4 = dg64_vel(p, ds_add_u(x, ds_mul_u(S1, w3)), c2);
+        const dsf x = ds_make(xh, xm), a1 = ds_make(c1.x, c1.y), b1 = ds_make(c1.z, c1.w);
+        const dsf w1 = dg_pair_vel<false, true>(p, kFull, x, ds_make(c0.x, c0.y), ds_make(c0.z, c0.w));
+        const dsf w2 = dg_pair_vel<false, true>(p, kFull, ds_add_u(x, ds_mul_u(S2, w1)), a1, b1);
+        const dsf w3 = dg_pair_vel<false, true>(p, kFull, ds_add_u(x, ds_mul_u(S2, w2)), a1, b1);
+        const dsf w4 = dg_pair_vel<false, true>(p, kFull, ds_add_u(x, ds_mul_u(S1, w3)), ds_make(c2.x, c2.y), ds_make(c2.z, c2.w));
         c0 = c2;
         const dsf s23 = ds_add_u(w2, w3);
         const dsf s = ds_add(ds_add_u(w1, w4), ds_make(2.0f * s23.h, 2.0f * s23.l));

@@ -6,6 +6,7 @@
 #include "advect.cuh"
 #include "batch.cuh"
 #include "capi_internal.cuh"
+#include "dg_pair.cuh"
 #include "dsfloat.cuh"
 
 namespace ftle {
@@ -137,19 +138,11 @@ __global__ void __launch_bounds__(32) k_advect_ds(AdvArgs a) {
   }
 }
 
-// Double gyre in 2D with two lanes per node: lane p = 0 carries x and evaluates sin/cos(pi f),
-// lane p = 1 carries y and evaluates sin/cos(pi y).  Both lanes run one instruction stream: the
-// argument is f = (a_p x + b_p) x with (a_p, b_p) = (a, 1 - 2a) for p = 0 and (0, 1) for p = 1,
-// so lane 1's argument is y and its slope is 1.  Each lane then needs only the partner's cosine
-// and slope (four floats by shuffle):
-//   u = -pi A sin(pi f) cos(pi y),  v = pi A sin(pi y) cos(pi f) f_x,
-// and updates its own coordinate.  The node's two float-float chains run on two lanes instead of
-// interleaving in one, which halves the instructions a lane issues per stage; the arithmetic is
-// the single-lane kernel's up to the order of the velocity product and of the final sum.
+// Double gyre in 2D with two lanes per node (dg_pair_vel): the node's two float-float chains run on two
+// lanes instead of interleaving in one, which halves the instructions a lane issues per stage.
 struct DsPairConst {
-  dsf piA;              // -pi A on lane 0, pi A on lane 1
-  dsf h, h2, h6, third;
-  unsigned int mask;    // the two lanes of this pair
+  dsf S2, S1, S6;       // -pi A (lane 0) or pi A (lane 1) times h/2, h, h/6
+  unsigned int mask;    // the lanes that step together
   int p;
 };
 
@@ -159,42 +152,30 @@ __device__ __forceinline__ DsPairConst ds_pair_const(const AdvArgs& a, bool whol
   DsPairConst K;
   K.p = threadIdx.x & 1;
   K.mask = whole_warp ? 0xffffffffu : 3u << (threadIdx.x & 30);
-  K.piA = ds_from_double((K.p ? kPi : -kPi) * a.p[0]);
-  K.h = ds_from_double(a.h);
-  K.h2 = ds_from_double(0.5 * a.h);
-  K.h6 = ds_from_double(a.h / 6.0);
-  K.third = ds_from_double(1.0 / 3.0);
+  const double s = (K.p ? kPi : -kPi) * a.p[0] * a.h;
+  K.S2 = ds_from_double(0.5 * s);
+  K.S1 = ds_from_double(s);
+  K.S6 = ds_from_double(s / 6.0);
   return K;
 }
 
-// hc times this lane's velocity component at y, with a(t) = ca: the scale (a stage's step
-// fraction times -pi A or pi A times the partner's slope) is formed while the sine and cosine
-// evaluate, so two products follow them on the dependency chain.
-__device__ __forceinline__ dsf ds_pair_dg_vel(const DsPairConst& K, const dsf& y, const dsf& ca, const dsf& hc) {
-  const dsf ap = K.p ? ds_make(0.f, 0.f) : ca;
-  const dsf bp = K.p ? ds_make(1.0f, 0.0f) : ds_add_f(ds_make(-2.0f * ca.h, -2.0f * ca.l), 1.0f);
-  const dsf t1 = ds_mul_u(ap, y);
-  const dsf f = ds_mul(ds_add_u(t1, bp), y);  // normalized: its high part is reduced by rint
-  const dsf fx = ds_add(ds_make(2.0f * t1.h, 2.0f * t1.l), bp);
-  const dsf fq = ds_make(__shfl_xor_sync(K.mask, fx.h, 1), __shfl_xor_sync(K.mask, fx.l, 1));
-  const dsf g = ds_make(K.p ? fq.h : 1.0f, K.p ? fq.l : 0.0f);
-  const dsf scale = ds_mul(ds_mul(K.piA, g), hc);
-  dsf sn, cs;
-  ds_sincospi(f, sn, cs);
-  const dsf cq = ds_make(__shfl_xor_sync(K.mask, cs.h, 1), __shfl_xor_sync(K.mask, cs.l, 1));
-  return ds_mul_u(ds_mul_u(sn, cq), scale);
+// x + h/6 (k1 + 2 k2 + 2 k3 + k4) from the stage velocities w without their factor.
+__device__ __forceinline__ dsf ds_pair_update(const DsPairConst& K, const dsf& x, const dsf& w1, const dsf& w2,
+                                              const dsf& w3, const dsf& w4) {
+  const dsf s23 = ds_add_u(w2, w3);
+  const dsf s = ds_add(ds_add_u(w1, w4), ds_make(2.0f * s23.h, 2.0f * s23.l));
+  return ds_add(x, ds_mul_u(K.S6, s));
 }
 
-// One RK4 step of this lane's coordinate, with a(t) at the step's start, middle and end:
-// d1 = h/2 k1, d2 = h/2 k2, d3 = h k3, e4 = h/6 k4, and x + (d1 + 2 d2 + d3) / 3 + e4.
+// One RK4 step of this lane's coordinate, with a(t) at the step's start, middle and end.
 __device__ __forceinline__ dsf ds_pair_dg_step(const DsPairConst& K, const dsf& x, const dsf& c0, const dsf& c1,
                                                const dsf& c2) {
-  const dsf d1 = ds_pair_dg_vel(K, x, c0, K.h2);
-  const dsf d2 = ds_pair_dg_vel(K, ds_add_u(x, d1), c1, K.h2);
-  const dsf d3 = ds_pair_dg_vel(K, ds_add_u(x, d2), c1, K.h);
-  const dsf e4 = ds_pair_dg_vel(K, ds_add_u(x, d3), c2, K.h6);
-  const dsf sum = ds_add(ds_add(d1, d3), ds_make(2.0f * d2.h, 2.0f * d2.l));
-  return ds_add(x, ds_add(ds_mul(sum, K.third), e4));
+  const dsf b1 = dg_pair_b(c1);
+  const dsf w1 = dg_pair_vel<false, false>(K.p, K.mask, x, c0, dg_pair_b(c0));
+  const dsf w2 = dg_pair_vel<false, false>(K.p, K.mask, ds_add_u(x, ds_mul_u(K.S2, w1)), c1, b1);
+  const dsf w3 = dg_pair_vel<false, false>(K.p, K.mask, ds_add_u(x, ds_mul_u(K.S2, w2)), c1, b1);
+  const dsf w4 = dg_pair_vel<false, false>(K.p, K.mask, ds_add_u(x, ds_mul_u(K.S1, w3)), c2, dg_pair_b(c2));
+  return ds_pair_update(K, x, w1, w2, w3, w4);
 }
 
 // Lane 0 of a pair writes the node's gradient record (both coordinates, from the partner).
@@ -507,34 +488,6 @@ __global__ void k_ds_coef_table(double t0, double h, double eps, double omega, i
   if (m <= 2 * nsteps) tab[m] = ds_from_double(eps * sin(omega * (t0 + 0.5 * h * (double)m)));
 }
 
-// ds_pair_dg_vel plus this lane's row of the velocity gradient in float (piA = pi A):
-//   lane 0, u = -pi A sin(pi f) cos(pi y):  du/dx = -pi^2 A f_x cos(pi f) cos(pi y),
-//                                          du/dy =  pi^2 A sin(pi f) sin(pi y);
-//   lane 1, v = pi A cos(pi f) sin(pi y) f_x:  dv/dx = pi A sin(pi y) (2 a cos(pi f) - pi f_x^2 sin(pi f)),
-//                                              dv/dy = pi^2 A cos(pi f) cos(pi y) f_x.
-__device__ __forceinline__ dsf ds_pair_dg_vel_tan(const DsPairConst& K, const dsf& y, const dsf& ca, const dsf& hc,
-                                                  float piA, float& gx, float& gy) {
-  const float kPiF = 3.14159265358979323846f;
-  const dsf ap = K.p ? ds_make(0.f, 0.f) : ca;
-  const dsf bp = K.p ? ds_make(1.0f, 0.0f) : ds_add_f(ds_make(-2.0f * ca.h, -2.0f * ca.l), 1.0f);
-  const dsf t1 = ds_mul_u(ap, y);
-  const dsf f = ds_mul(ds_add_u(t1, bp), y);
-  const dsf fx = ds_add(ds_make(2.0f * t1.h, 2.0f * t1.l), bp);
-  const dsf fq = ds_make(__shfl_xor_sync(K.mask, fx.h, 1), __shfl_xor_sync(K.mask, fx.l, 1));
-  const dsf g = ds_make(K.p ? fq.h : 1.0f, K.p ? fq.l : 0.0f);
-  const dsf scale = ds_mul(ds_mul(K.piA, g), hc);
-  dsf sn, cs;
-  ds_sincospi(f, sn, cs);
-  const dsf cq = ds_make(__shfl_xor_sync(K.mask, cs.h, 1), __shfl_xor_sync(K.mask, cs.l, 1));
-  const float sq = __shfl_xor_sync(K.mask, sn.h, 1);
-  const float S = sn.h, C = cs.h, Cq = cq.h, fo = fx.h, fp = fq.h;
-  const float gx0 = -kPiF * piA * fo * C * Cq, gy0 = kPiF * piA * S * sq;
-  const float gx1 = piA * S * fmaf(2.0f * ca.h, Cq, -kPiF * fp * fp * sq), gy1 = kPiF * piA * Cq * C * fp;
-  gx = K.p ? gx1 : gx0;
-  gy = K.p ? gy1 : gy0;
-  return ds_mul_u(ds_mul_u(sn, cq), scale);
-}
-
 // This lane's tangent row times the stage gradient: (g . J)_p with J's rows on lanes 0 and 1.
 __device__ __forceinline__ float2 ds_pair_tan_row(const DsPairConst& K, float gx, float gy, float2 jr) {
   const float2 jq = make_float2(__shfl_xor_sync(K.mask, jr.x, 1), __shfl_xor_sync(K.mask, jr.y, 1));
@@ -546,19 +499,19 @@ __device__ __forceinline__ float2 ds_pair_tan_row(const DsPairConst& K, float gx
 __device__ __forceinline__ dsf ds_pair_dg_step_tan(const DsPairConst& K, const dsf& x, float2& jr, const dsf& c0,
                                                    const dsf& c1, const dsf& c2, float piA, float h) {
   float gx, gy;
-  const dsf d1 = ds_pair_dg_vel_tan(K, x, c0, K.h2, piA, gx, gy);
+  const dsf b1 = dg_pair_b(c1);
+  const dsf w1 = dg_pair_vel<true, false>(K.p, K.mask, x, c0, dg_pair_b(c0), piA, &gx, &gy);
   const float2 k1 = ds_pair_tan_row(K, gx, gy, jr);
-  const dsf d2 = ds_pair_dg_vel_tan(K, ds_add_u(x, d1), c1, K.h2, piA, gx, gy);
+  const dsf w2 = dg_pair_vel<true, false>(K.p, K.mask, ds_add_u(x, ds_mul_u(K.S2, w1)), c1, b1, piA, &gx, &gy);
   const float2 k2 = ds_pair_tan_row(K, gx, gy, make_float2(fmaf(0.5f * h, k1.x, jr.x), fmaf(0.5f * h, k1.y, jr.y)));
-  const dsf d3 = ds_pair_dg_vel_tan(K, ds_add_u(x, d2), c1, K.h, piA, gx, gy);
+  const dsf w3 = dg_pair_vel<true, false>(K.p, K.mask, ds_add_u(x, ds_mul_u(K.S2, w2)), c1, b1, piA, &gx, &gy);
   const float2 k3 = ds_pair_tan_row(K, gx, gy, make_float2(fmaf(0.5f * h, k2.x, jr.x), fmaf(0.5f * h, k2.y, jr.y)));
-  const dsf e4 = ds_pair_dg_vel_tan(K, ds_add_u(x, d3), c2, K.h6, piA, gx, gy);
+  const dsf w4 = dg_pair_vel<true, false>(K.p, K.mask, ds_add_u(x, ds_mul_u(K.S1, w3)), c2, dg_pair_b(c2), piA, &gx, &gy);
   const float2 k4 = ds_pair_tan_row(K, gx, gy, make_float2(fmaf(h, k3.x, jr.x), fmaf(h, k3.y, jr.y)));
   const float h6 = h * (1.0f / 6.0f);
   jr.x = fmaf(h6, fmaf(2.0f, k2.x + k3.x, k1.x + k4.x), jr.x);
   jr.y = fmaf(h6, fmaf(2.0f, k2.y + k3.y, k1.y + k4.y), jr.y);
-  const dsf sum = ds_add(ds_add(d1, d3), ds_make(2.0f * d2.h, 2.0f * d2.l));
-  return ds_add(x, ds_add(ds_mul(sum, K.third), e4));
+  return ds_pair_update(K, x, w1, w2, w3, w4);
 }
 
 // The join of a node's runs (lanes grp .. grp + 2 kSegments - 1, K.mask covering them): with x the
@@ -600,7 +553,7 @@ __device__ __forceinline__ void ds_runs_join_store(const AdvArgs& a, const DsPai
 // Persistent blocks of 128 threads; a node takes 2 kSegments lanes of one warp: run j on lanes
 // 2j (x) and 2j + 1 (y).  `coef` holds the coefficient table (k_ds_coef_table).  Held to eight
 // 128-thread blocks per SM (64 registers): 1.017 -> 0.977 ms on the 2D workload's 11,222 nodes,
-// against 72 registers and seven blocks.
+// against 72 registers and seven blocks; with dg_pair_vel 1.28 -> 1.11 ms under the profiler.
 template <typename CT>
 __global__ void __launch_bounds__(128, 8) k_refine_runs_dg(AdvArgs a, const dsf* __restrict__ coef) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -732,9 +685,10 @@ __global__ void __launch_bounds__(32) k_batch_advect_ds(const BatchInst* __restr
 // Batched run-parallel re-advection (2D double gyre, compensated flowmaps with run-boundary
 // states): a half-warp per (instance, node) pair, run j on its lanes 2j and 2j + 1.  The two
 // halves of a warp may belong to instances with different steps, so every shuffle names only its
-// half.  Each run forms its time coefficients a(t) = eps sin(omega t) by turning
-// (sin, cos)(omega t) from its own first half step through omega h/2 per half step.
-__global__ void __launch_bounds__(128) k_batch_refine_runs_dg(const BatchInst* __restrict__ insts, const int2* pairs,
+// half.  Each run forms its time coefficients a(t) = eps sin(omega t) from its own first half step.
+// 24 instances (3.4 M nodes): 3.57 ms with (sin, cos)(omega t) turned in float-float at each half step
+// and the earlier velocity (96 registers), 3.05 ms now at 80 registers, 2.98 at 64.
+__global__ void __launch_bounds__(128, 8) k_batch_refine_runs_dg(const BatchInst* __restrict__ insts, const int2* pairs,
                                                               const unsigned long long* count) {
   const int lane = threadIdx.x & 31;
   const int run = (lane >> 1) & (kSegments - 1);
@@ -758,24 +712,25 @@ __global__ void __launch_bounds__(128) k_batch_refine_runs_dg(const BatchInst* _
       const float2 c = a.seg[(int64_t)(run - 1) * a.seg_stride + K.p * a.n_mesh + i];
       x = ds_make(c.x, c.y);
     }
-    const dsf eps = ds_from_double(a.p[1]);
-    const dsf rs = ds_from_double(sin(0.5 * a.p[2] * a.h)), rc = ds_from_double(cos(0.5 * a.p[2] * a.h));
-    const double t_start = a.t0 + a.h * (double)(run * L);
-    dsf sw = ds_from_double(sin(a.p[2] * t_start)), cw = ds_from_double(cos(a.p[2] * t_start));
+    // a(t) = eps sin(omega t) from half step to half step by its differences: a_{m+1} = a_m + e_{m+1},
+    // e_{m+1} = e_m - 4 sin^2(omega h/4) a_m (exact for a sine; over a run's few hundred half steps
+    // the float-float roundings add up to ~3e-14)
+    const double half = 0.5 * a.p[2] * a.h, t_start = a.t0 + a.h * (double)(run * L);
+    const double sq = sin(0.5 * half), a_start = a.p[1] * sin(a.p[2] * t_start);
+    const dsf kap = ds_from_double(-4.0 * sq * sq);
+    dsf c2 = ds_from_double(a_start);
+    dsf e = ds_from_double(2.0 * a.p[1] * sq * cos(a.p[2] * t_start - 0.5 * half));  // a_0 - a_{-1}
     auto advance = [&]() {
-      const dsf s2 = ds_add(ds_mul(sw, rc), ds_mul(cw, rs));
-      cw = ds_add(ds_mul(cw, rc), ds_neg(ds_mul(sw, rs)));
-      sw = s2;
+      e = ds_add(e, ds_mul_u(kap, c2));
+      c2 = ds_add(c2, e);
     };
     float2 jr = make_float2(K.p == 0 ? 1.0f : 0.0f, K.p == 0 ? 0.0f : 1.0f);
-    dsf c2 = ds_mul(eps, sw);
     for (int s = 0; s < L; ++s) {  // every lane of the half-warp runs L steps; past nsteps discarded
       const bool live = run * L + s < a.nsteps;
       const dsf c0 = c2;
       advance();
-      const dsf c1 = ds_mul(eps, sw);
+      const dsf c1 = c2;
       advance();
-      c2 = ds_mul(eps, sw);
       float2 jn = jr;
       const dsf xn = ds_pair_dg_step_tan(K, x, jn, c0, c1, c2, piA, h);
       if (live) {

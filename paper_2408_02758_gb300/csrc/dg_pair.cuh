@@ -1,0 +1,53 @@
+// The double gyre's velocity in float-float with two lanes of a warp per node: lane p = 0 carries x and
+// evaluates (sin, cos)(pi f), lane p = 1 carries y and evaluates (sin, cos)(pi y).  Both run one
+// instruction stream: the argument is f = z + a_p z (z - 2) with a_0 = a(t) and a_1 = 0, so lane 1's is
+// y and its slope 1.  Each lane needs only the partner's cosine and slope (four floats by shuffle):
+//   u = -pi A sin(pi f) cos(pi y),  v = pi A sin(pi y) cos(pi f) f_x.
+#pragma once
+
+#include "dsfloat.cuh"
+
+namespace ftle {
+
+// b = 1 - 2a.
+__device__ __forceinline__ dsf dg_pair_b(dsf a) {  // |2a| <= 1 where |eps| <= 1/2, else within an ulp of a's
+  const dsf b = ds_make(-2.0f * a.h, -2.0f * a.l);
+  return ds_add_f(b, 1.0f);
+}
+
+// This lane's velocity component at z without its factor (-pi A, pi A), b = 1 - 2a.  Error about
+// 2e-15 rms.  With TAN also this lane's row of the velocity gradient in float (piA = pi A):
+//   lane 0:  du/dx = -pi^2 A f_x cos(pi f) cos(pi y),  du/dy = pi^2 A sin(pi f) sin(pi y);
+//   lane 1:  dv/dx = pi A sin(pi y) (2 a cos(pi f) - pi f_x^2 sin(pi f)),
+//            dv/dy = pi^2 A cos(pi f) cos(pi y) f_x.
+// mask: the lanes that reach the shuffles together.  IN: z stays within the domain [0, 2] x [0, 1] (but
+// for a stage's rounding), so z - 2 takes a Fast2Sum and f its sine table's range.
+template <bool TAN, bool IN>
+__device__ __forceinline__ dsf dg_pair_vel(int p, unsigned int mask, const dsf& z, const dsf& a, const dsf& b,
+                                           float piA = 0.f, float* gx = nullptr, float* gy = nullptr) {
+  const dsf t1 = ds_mul_u(ds_make(p ? 0.f : a.h, p ? 0.f : a.l), z);
+  dsf z2;  // z - 2, normalized for the nodes near the wall at 2
+  if constexpr (IN)
+    z2 = ds_fast(-2.0f, z.h);
+  else
+    two_sum(-2.0f, z.h, z2.h, z2.l);
+  z2 = ds_fast(z2.h, __fadd_rn(z2.l, z.l));
+  dsf f = ds_add_u(z, ds_mul_u(t1, z2));
+  if constexpr (!IN)
+    if (!(fabsf(f.h) < 4096.0f)) f = ds_fast(f.h - 2.0f * rintf(0.5f * f.h), f.l);  // whole periods out
+  const dsf fx = ds_add_u(ds_make(2.0f * t1.h, 2.0f * t1.l), b);
+  const float gh = __shfl_xor_sync(mask, fx.h, 1), gl = __shfl_xor_sync(mask, fx.l, 1);
+  dsf sn, cs;
+  ds_sincospi_fold(f, sn, cs);
+  const dsf cq = ds_make(__shfl_xor_sync(mask, cs.h, 1), __shfl_xor_sync(mask, cs.l, 1));
+  if constexpr (TAN) {
+    const float kPiF = 3.14159265358979323846f;
+    const float sq = __shfl_xor_sync(mask, sn.h, 1);
+    const float pc = kPiF * piA * cs.h * cq.h, ps = piA * sn.h;
+    *gx = p ? ps * fmaf(2.0f * a.h, cq.h, -kPiF * gh * gh * sq) : -pc * fx.h;
+    *gy = p ? pc * gh : kPiF * ps * sq;
+  }
+  return ds_mul_u(ds_mul_u(sn, cq), ds_make(p ? gh : 1.0f, p ? gl : 0.0f));
+}
+
+}  // namespace ftle
