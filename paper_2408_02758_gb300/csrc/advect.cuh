@@ -1194,6 +1194,87 @@ __device__ __forceinline__ void dg_walk(const AdvArgs& a, const float2* tab, int
   w.end(a, i, stride, active);
 }
 
+// The plain float double-gyre step of one node or of two (the bits of rk4_step<.., P32>).
+template <class V>
+__device__ __forceinline__ void dg32_vel(float piA, float a, float b, V x, V y, V& u, V& v) {
+  const V g = vfma(vsplat<V>(a), x, vsplat<V>(b));
+  V sf, cf, sy, cy;
+  vsincospi(vmul(g, x), sf, cf);
+  vsincospi(y, sy, cy);
+  u = vmul(vmul(vsplat<V>(-piA), sf), cy);
+  v = vmul(vmul(vmul(vsplat<V>(piA), cf), sy), vfma(vsplat<V>(2.0f * a), x, vsplat<V>(b)));
+}
+
+// k_advect for plain float double-gyre flowmaps, N nodes per thread.  Full sines and cosines at every
+// stage: the paired lanes halve the FP32 instructions' issue slots beside the quarter turns' integer
+// work (144 integer operations against 146 paired ones for two nodes, which hold both pipes now).
+// 512 x 256 nodes, 1000 steps: 955 us with one node per thread in equal blocks of eight warps (some SMs
+// held four of them, others three), 902 with one node and blocks evened out, 842 with two nodes.
+template <int N, typename CT>
+__global__ void __launch_bounds__(256, N == 2 ? 2 : 4) k_advect_dg32(AdvArgs a) {
+  using V = typename std::conditional<N == 2, float2, float>::type;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* tab = reinterpret_cast<float2*>(smem_raw);
+  const int warps = blockDim.x >> 5;
+  const int64_t tiles = (a.n + 32 * N - 1) / (32 * N), per_round = (int64_t)gridDim.x * warps;
+  const float piA = (float)(kPi * a.p[0]);
+  bool valid = false;
+  for (int64_t r0 = 0; r0 < tiles; r0 += per_round) {  // the same rounds for every warp of the block
+    const int64_t tile = r0 + (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int64_t i = tile * 32 * N + (threadIdx.x & 31);
+    const bool any = i < a.n, two = N == 2 && i + 32 < a.n;
+    V x[2];
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+#pragma unroll
+      for (int d = 0; d < 2; ++d)
+        vset(x[d], q, any ? (float)load_coord<CT>(a.coords, d * a.n_mesh + (q && two ? i + 32 : i)) : 0.0f);
+    auto store = [&](void* base) {
+      float* o = reinterpret_cast<float*>(base);
+#pragma unroll
+      for (int q = 0; q < N; ++q)
+        if (any && (q == 0 || two)) {
+          o[i + 32 * q] = vget(x[0], q);
+          o[a.n_mesh + i + 32 * q] = vget(x[1], q);
+        }
+    };
+    int ck_left = a.ckpt_every, ck_slot = 1;
+    if (a.ckpt) store(a.ckpt);
+    for (int k0 = 0; k0 < a.nsteps; k0 += kAdvChunk) {
+      const int k1 = min(a.nsteps, k0 + kAdvChunk);
+      if (!(valid && a.nsteps <= kAdvChunk)) {
+        __syncthreads();
+        build_table<FTLE_FLOW_DOUBLE_GYRE, P32>(a, tab, nullptr, k0, k1);
+        __syncthreads();
+        valid = true;
+      }
+      if (!any) continue;
+      float a0 = tab[0].x;
+      for (int k = k0; k < k1; ++k) {
+        const float a1 = tab[2 * (k - k0) + 1].x, a2 = tab[2 * (k - k0) + 2].x;
+        const float b0 = fmaf(-2.f, a0, 1.f), b1 = fmaf(-2.f, a1, 1.f), b2 = fmaf(-2.f, a2, 1.f);
+        V k1v[2], k2v[2], k3v[2], k4v[2];
+        const V h2 = vsplat<V>(a.h2_32), h = vsplat<V>(a.h32);
+        dg32_vel(piA, a0, b0, x[0], x[1], k1v[0], k1v[1]);
+        dg32_vel(piA, a1, b1, vfma(h2, k1v[0], x[0]), vfma(h2, k1v[1], x[1]), k2v[0], k2v[1]);
+        dg32_vel(piA, a1, b1, vfma(h2, k2v[0], x[0]), vfma(h2, k2v[1], x[1]), k3v[0], k3v[1]);
+        dg32_vel(piA, a2, b2, vfma(h, k3v[0], x[0]), vfma(h, k3v[1], x[1]), k4v[0], k4v[1]);
+#pragma unroll
+        for (int d = 0; d < 2; ++d)
+          x[d] = vfma(vsplat<V>(a.h6_32),
+                      vfma(vsplat<V>(2.f), vadd(k2v[d], k3v[d]), vadd(k1v[d], k4v[d])), x[d]);
+        a0 = a2;
+        if (a.ckpt && --ck_left == 0) {
+          ck_left = a.ckpt_every;
+          store(reinterpret_cast<char*>(a.ckpt) + (int64_t)ck_slot * a.ckpt_stride_bytes);
+          ++ck_slot;
+        }
+      }
+    }
+    store(a.out);
+  }
+}
+
 // Up to two ABC nodes of a thread (V = float2: nodes i and i + stride, the second inside the mesh when
 // two is set) from their coordinates to their records.
 template <class V, typename CT>

@@ -9,8 +9,9 @@ int launch_advect_typed(int prec, int out, const AdvArgs& args, int grid, int bl
                         cudaStream_t stream) {
   if (prec == P64 && out == O64) {
     k_advect<KIND, DIM, P64, O64, CT><<<grid, block, smem, stream>>>(args);
-  } else if (prec == P32 && out == O32) {
-    k_advect<KIND, DIM, P32, O32, CT><<<grid, block, smem, stream>>>(args);
+  } else if (KIND != FTLE_FLOW_DOUBLE_GYRE && prec == P32 && out == O32) {
+    if constexpr (KIND != FTLE_FLOW_DOUBLE_GYRE)  // the double gyre: k_advect_dg32
+      k_advect<KIND, DIM, P32, O32, CT><<<grid, block, smem, stream>>>(args);
   } else if (prec == P32C && out == O32PAIR) {
     constexpr bool kAbc = KIND == FTLE_FLOW_ABC;
     if (kAbc && args.rot_safe)

@@ -479,10 +479,11 @@ int run_advect(const ftle_mesh* m, const ftle_flow* fl, double t0, double T, dou
     if (rc) return rc;
     a.dg64 = 1;
   }
-  if (prec == P32C && a.dg_carry)
-    return launch_advect_dg_carry(m->coord_fp64 != 0, a, L.advect_shape ? L.advect_block : 0, L.advect_bps, s);
-  if (prec == P32C && a.carry_ok && a.abc_refresh > 1)
-    return launch_advect_abc_carry(m->coord_fp64 != 0, a, L.advect_shape ? L.advect_block : 0, L.advect_bps, s);
+  const bool dg = fl->kind == FTLE_FLOW_DOUBLE_GYRE, c64 = m->coord_fp64 != 0;
+  const int shape = L.advect_shape ? L.advect_block : 0;
+  if (prec == P32 && dg) return launch_advect_dg32(c64, a, shape, L.advect_bps, s);
+  if (prec == P32C && a.dg_carry) return launch_advect_dg_carry(c64, a, shape, L.advect_bps, s);
+  if (prec == P32C && a.carry_ok && a.abc_refresh > 1) return launch_advect_abc_carry(c64, a, shape, L.advect_bps, s);
   int block = L.advect_block;
   if (prec == P64 && block > 128) block = 128;
   // by default a grid of 8192 / block blocks per SM (32 of 256 threads), more than fit at once:

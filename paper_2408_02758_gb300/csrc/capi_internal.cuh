@@ -64,6 +64,34 @@ int launch_advect_dg(int prec, int out, bool coord64, const AdvArgs& args, int g
                      size_t smem, cudaStream_t stream);
 int launch_advect_abc(int prec, int out, bool coord64, const AdvArgs& args, int grid, int block,
                       size_t smem, cudaStream_t stream);
+// Launch shape of the kernels that take one or two nodes per thread (32 or 64 consecutive ones per warp):
+//   up to one warp per SM sub-partition one node per thread, which has the shorter chain per step, in
+//   blocks of four warps, one on each sub-partition;
+//   while two nodes per thread fit at once (16 warps per SM) two blocks per SM of equal size, so that
+//   the SMs differ by a warp;
+//   beyond that blocks of four warps, which even out the last round, or, from `eight` warps per SM on,
+//   of eight, which make their coefficient tables half as often.
+// block > 0: that many threads per block; blocks_per_sm > 0: at most that many blocks per SM.
+struct NodeShape {
+  bool two;
+  int grid, block;
+};
+inline NodeShape node_shape(int64_t n, int block, int blocks_per_sm, int64_t eight) {
+  const int64_t sms = device_sm_count() > 0 ? device_sm_count() : 1;
+  NodeShape S;
+  S.two = n > sms * 4 * 32;
+  const int64_t tile = S.two ? 64 : 32, tiles = (n + tile - 1) / tile, per_sm = (tiles + sms - 1) / sms;
+  int64_t warps = block / 32;
+  if (block <= 0) warps = !S.two ? 4 : per_sm <= 16 ? (per_sm + 1) / 2 : per_sm < eight ? 4 : 8;
+  const int64_t need = (tiles + warps - 1) / warps;
+  const int64_t cap = blocks_per_sm > 0 ? sms * blocks_per_sm : need;
+  S.grid = (int)(need < cap ? need : cap);
+  S.block = 32 * (int)warps;
+  return S;
+}
+
+// Plain float double-gyre advection (block, blocks_per_sm: node_shape).
+int launch_advect_dg32(bool coord64, const AdvArgs& args, int block, int blocks_per_sm, cudaStream_t s);
 // Compensated advection with carried sines and cosines (AdvArgs::dg_carry, carry_ok); block 0: the
 // launch shape of its own choice, blocks_per_sm 0: no limit on the grid.
 int launch_advect_abc_carry(bool coord64, const AdvArgs& args, int block, int blocks_per_sm, cudaStream_t s);

@@ -100,8 +100,9 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
-// One node's float or two nodes' lanes: the same operations, rounded alike and never contracted
-// further, so that a step written on them gives a node the same bits either way.
+// One node's float or two nodes' lanes: the same operations, rounded alike (the compiler contracts a
+// product and the sum it feeds in either form), so that a step written on them gives a node the
+// same bits either way; the tests compare them.
 template <class V>
 __device__ __forceinline__ V vsplat(float x);
 template <>
@@ -109,8 +110,8 @@ __device__ __forceinline__ float vsplat<float>(float x) { return x; }
 template <>
 __device__ __forceinline__ float2 vsplat<float2>(float x) { return f2(x); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
 __device__ __forceinline__ float vneg(float a) { return -a; }
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
@@ -146,6 +147,26 @@ __device__ __forceinline__ void fsincos_c(float xh, float xl, float& s, float& c
   const float ps = fmaf(fmaf(fmaf(kRAD_S[3], z, kRAD_S[2]), z, kRAD_S[1]), z, kRAD_S[0]) * rh;
   const float pc = fmaf(fmaf(fmaf(fmaf(kRAD_C[4], z, kRAD_C[3]), z, kRAD_C[2]), z, kRAD_C[1]), z, kRAD_C[0]);
   quarter_turn(t, fmaf(rl, pc, ps), fmaf(-rl, ps, pc), s, c);
+}
+
+// fsincospi of one node or of two.
+template <class V>
+__device__ __forceinline__ void vsincospi(V x, V& s, V& c) {
+  const V t = vfma(x, vsplat<V>(2.0f), vsplat<V>(kRoundMagic));
+  const V k = vadd(t, vsplat<V>(-kRoundMagic));
+  const V r = vfma(k, vsplat<V>(-0.5f), x);
+  const V z = vmul(r, r);
+  const V ps = vmul(vfma(vfma(vfma(vsplat<V>(kPI_S[3]), z, vsplat<V>(kPI_S[2])), z, vsplat<V>(kPI_S[1])), z,
+                         vsplat<V>(kPI_S[0])), r);
+  const V pc = vfma(vfma(vfma(vfma(vsplat<V>(kPI_C[4]), z, vsplat<V>(kPI_C[3])), z, vsplat<V>(kPI_C[2])), z,
+                         vsplat<V>(kPI_C[1])), z, vsplat<V>(kPI_C[0]));
+#pragma unroll
+  for (int q = 0; q < (int)(sizeof(V) / sizeof(float)); ++q) {
+    float a, b;
+    quarter_turn(vget(t, q), vget(ps, q), vget(pc, q), a, b);
+    vset(s, q, a);
+    vset(c, q, b);
+  }
 }
 
 // fsincos_c of one node or of two.
