@@ -29,7 +29,8 @@
 
 namespace ftle {
 
-constexpr int kAdjBlock = 64;
+constexpr int kAdjBlock = 128;    // threads per block, at most
+constexpr int kAdjBlockMin = 64;  // ... where longer segments' states would not leave room for four blocks
 
 // ------------------------------------------------------------------- 1. FTLE-map adjoint
 
@@ -101,61 +102,61 @@ __global__ void __launch_bounds__(128) k_ftle_adjoint_gather(GradArgs g, const d
 
 // ---------------------------------------------------------------- 2. RK4 discrete adjoint
 
-struct DgDer {
-  float u0, u1;              // velocity
-  float j01, j10, j11;       // du/dx (j00 = -j11: the flow is divergence-free)
-  float pA0, pA1;            // du/dA / pi
-  float q0, q1;              // du/deps = s q, du/domega = eps t c q
+// What the reverse sweep needs of a stage: the four products of the sines and cosines of pi f and pi y,
+// the slope f_x, and d(f)/da = x^2 - 2x and its derivative 2x - 2.
+struct DgStage {
+  float scy, ccy, csy, ssy, fx, g1, g2;
 };
 
-// Double-gyre velocity and derivatives at a point with abscissa x, from the slope f_x of the
-// stream function's argument and (sin, cos) of pi f and of pi y there; coefficient a = eps s.
-// The four products of the sines and cosines are formed once and shared.
-__device__ __forceinline__ DgDer dg_derivs_sc(float piA, float a, float fx, float x, float sf, float cf, float sy,
-                                              float cy) {
-  const float kPiF = 3.14159265358979323846f;
-  DgDer d;
-  const float scy = sf * cy, ccy = cf * cy, csy = cf * sy, ssy = sf * sy;
-  const float t1 = csy * fx;
-  const float pi2A = kPiF * piA;
-  d.u0 = -piA * scy;
-  d.u1 = piA * t1;
-  d.j01 = pi2A * ssy;
-  d.j10 = piA * fmaf(-kPiF * ssy, fx * fx, csy * 2.0f * a);
-  d.j11 = pi2A * (ccy * fx);
-  d.pA0 = -scy;
-  d.pA1 = t1;
-  const float g1 = fmaf(x, x, -2.0f * x), g2 = fmaf(2.0f, x, -2.0f);
-  d.q0 = -pi2A * (ccy * g1);
-  d.q1 = piA * fmaf(-kPiF * ssy * g1, fx, csy * g2);
+__device__ __forceinline__ DgStage dg_stage(float sf, float cf, float sy, float cy, float fx, float g2) {
+  DgStage d;
+  d.scy = sf * cy, d.ccy = cf * cy, d.csy = cf * sy, d.ssy = sf * sy;
+  d.fx = fx, d.g2 = g2;
+  d.g1 = fmaf(0.25f * g2, g2, -1.0f);
   return d;
 }
 
 // ... at (x, y) with coefficients a, b = 1 - 2a, evaluating the sines and cosines.
-__device__ __forceinline__ DgDer dg_derivs32(float piA, float a, float b, float x, float y) {
-  const float f = fmaf(a, x, b) * x;
+__device__ __forceinline__ DgStage dg_stage_full(float a, float b, float x, float y) {
   float sf, cf, sy, cy;
-  fsincospi(f, sf, cf);
+  fsincospi(fmaf(a, x, b) * x, sf, cf);
   fsincospi(y, sy, cy);
-  return dg_derivs_sc(piA, a, fmaf(2.0f * a, x, b), x, sf, cf, sy, cy);
+  return dg_stage(sf, cf, sy, cy, fmaf(2.0f * a, x, b), fmaf(2.0f, x, -2.0f));
 }
 
-// ... at the stage point (xk + dx, yk + dy) of a step whose first stage point is (xk, yk), with
-// (sin, cos) of pi f and pi y there turned from stage one's pairs by the small angles, as the
-// forward step does (e1 = 2 (xk - 1), dg = (a_s - a_0) xk (xk - 2)).  `mx` collects the larger
-// angle; past kRotMax the caller evaluates the stage in full.
-__device__ __forceinline__ DgDer dg_derivs32_rot(float piA, float as, float e1, float dg, float dx, float dy,
-                                                 float sf0, float cf0, float sy0, float cy0, float xs, float& mx) {
+// ... at the stage point (xk + dx, .) of a step whose first stage point is (xk, yk), with (sin, cos)
+// of pi f and pi y turned from stage one's pairs (s0, c0: lanes pi f, pi y) by the small angles, as
+// the forward step does (e1 = 2 (xk - 1), dg = (a_s - a_0) xk (xk - 2), ty pi times the y increment).
+// `mx` collects the larger angle; past kRotMax the caller evaluates the stage in full.
+template <bool CHECK>
+__device__ __forceinline__ DgStage dg_stage_rot(float as, float e1, float dg, float dx, float ty, float2 s0, float2 c0,
+                                                float& mx) {
   const float kPiF = 3.14159265358979323846f;
   const float w = fmaf(as, e1 + dx, 1.0f);
-  const float tf = kPiF * fmaf(dx, w, dg), ty = kPiF * dy;
-  mx = fmaxf(mx, fmaxf(fabsf(tf), fabsf(ty)));
-  float2 s, c;  // lanes: pi f, pi y
-  rotate_small2(make_float2(sf0, sy0), make_float2(cf0, cy0), make_float2(tf, ty), s, c);
-  return dg_derivs_sc(piA, as, fmaf(as, dx, w), xs, s.x, c.x, s.y, c.y);
+  const float tf = kPiF * fmaf(dx, w, dg);
+  if constexpr (CHECK) mx = fmaxf(mx, fmaxf(fabsf(tf), fabsf(ty)));
+  float2 s, c;
+  rotate_small2(s0, c0, make_float2(tf, ty), s, c);
+  return dg_stage(s.x, c.x, s.y, c.y, fmaf(as, dx, w), fmaf(2.0f, dx, e1));
 }
 
-// Segment table per half step: (a, b_l) of the forward kernel, sin(omega t), t cos(omega t).
+// Reverse of one stage: for its adjoint kb, J^T kb (returned) and the parameter terms P^T kb added to
+// s0 (du/dA), s1 (eps), s2 (omega).  With L = pi^2 A kb, N = pi A cos(pi f) sin(pi y) kb_y and
+// M = cos cos L_x + sin sin f_x L_y, the x component is 2a N - f_x M and the common factor of the eps and
+// omega terms g2 N - g1 M: two thirds of the products that J and P formed apart would take.
+// tc: (a, ., sin(omega t), eps t cos(omega t)).
+__device__ __forceinline__ float2 dg_reverse(const DgStage& d, float2 kb, const float4& tc, float piA, float pi2A,
+                                             float& s0, float& s1, float& s2) {
+  const float Lx = pi2A * kb.x, fl = d.fx * (pi2A * kb.y);
+  const float M = fmaf(d.ccy, Lx, d.ssy * fl), N = d.csy * (piA * kb.y);
+  const float qk = fmaf(d.g2, N, -(d.g1 * M));
+  s0 = fmaf(-d.scy, kb.x, fmaf(d.csy * d.fx, kb.y, s0));
+  s1 = fmaf(tc.z, qk, s1);
+  s2 = fmaf(tc.w, qk, s2);
+  return make_float2(fmaf(2.0f * tc.x, N, -(d.fx * M)), fmaf(d.ssy, Lx, d.ccy * fl));
+}
+
+// Segment table per half step: (a, b_l) of the forward kernel, sin(omega t), eps t cos(omega t).
 // The sine and cosine take dg_coef's reduction: u = omega t / pi in double, then sinpi and cospi
 // of u - rint(u) in float, so no double transcendental runs (GB300's FP64 rate is low, and every
 // block rebuilds the table for every segment).
@@ -174,10 +175,13 @@ __device__ __forceinline__ void build_adj_table(const AdvArgs& a, float4* tab, i
       sr = -sr;
       cr = -cr;
     }
-    tab[m] = make_float4(c.x, c.y, sr, (float)t * cr);
+    tab[m] = make_float4(c.x, c.y, sr, (float)a.p[1] * ((float)t * cr));
   }
 }
 
+// Bound by instruction issue: the recomputed forward step and the reverse of four stages, with the segment's
+// states in shared memory (8 bytes a step and thread, so 16 to 20 warps per SM).  512 x 256 nodes,
+// T = 5, 500 steps: 850 us; 1002 with J^T and P^T formed apart and the angles checked at each stage.
 template <int PREC, int OUT>
 __global__ void __launch_bounds__(kAdjBlock) k_adjoint_rk4(AdvArgs a, const float* __restrict__ phibar,
                                                            double* __restrict__ partial) {
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adjoint_rk4(AdvArgs a, const floa
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = i < a.n;
   const float piA = (float)(kPi * a.p[0]);
-  const float eps = (float)a.p[1];
+  const float pi2A = 3.14159265358979323846f * piA;
   float lam0 = active ? phibar[i] : 0.f, lam1 = active ? phibar[a.n_mesh + i] : 0.f;
   // the forward kernel's choice between the checked and the unchecked step (dg_node_safe), so
   // the recomputed states are the forward's
@@ -247,55 +251,57 @@ __global__ void __launch_bounds__(kAdjBlock) k_adjoint_rk4(AdvArgs a, const floa
       // reverse the segment's steps
       float s0 = 0.f, s1 = 0.f, s2 = 0.f;
       const float h = a.h32, h2 = a.h2_32, h6 = a.h6_32, h3 = 2.0f * a.h6_32;
-      for (int k = k1 - 1; k >= k0; --k) {
-        const float2 xk = states[(k - k0) * blockDim.x + threadIdx.x];
-        const int m = 2 * (k - k0);
-        const float4 t0 = tab[m], t1 = tab[m + 1], t2 = tab[m + 2];
-        const float b0 = fmaf(-2.f, t0.x, 1.f), b1 = fmaf(-2.f, t1.x, 1.f), b2 = fmaf(-2.f, t2.x, 1.f);
-        // stage points (float); stages two to four turn stage one's sines and cosines
-        float sf0, cf0, sy0, cy0;
-        fsincospi(fmaf(t0.x, xk.x, b0) * xk.x, sf0, cf0);
-        fsincospi(xk.y, sy0, cy0);
-        const DgDer d1 = dg_derivs_sc(piA, t0.x, fmaf(2.0f * t0.x, xk.x, b0), xk.x, sf0, cf0, sy0, cy0);
-        const float e1 = fmaf(2.0f, xk.x, -2.0f), g0 = xk.x * (xk.x - 2.0f);
-        const float dg1 = (t1.x - t0.x) * g0, dg2 = (t2.x - t0.x) * g0;
-        float mx = 0.0f;
-        const float y2x = fmaf(h2, d1.u0, xk.x), y2y = fmaf(h2, d1.u1, xk.y);
-        DgDer d2 = dg_derivs32_rot(piA, t1.x, e1, dg1, y2x - xk.x, y2y - xk.y, sf0, cf0, sy0, cy0, y2x, mx);
-        const float y3x = fmaf(h2, d2.u0, xk.x), y3y = fmaf(h2, d2.u1, xk.y);
-        DgDer d3 = dg_derivs32_rot(piA, t1.x, e1, dg1, y3x - xk.x, y3y - xk.y, sf0, cf0, sy0, cy0, y3x, mx);
-        const float y4x = fmaf(h, d3.u0, xk.x), y4y = fmaf(h, d3.u1, xk.y);
-        DgDer d4 = dg_derivs32_rot(piA, t2.x, e1, dg2, y4x - xk.x, y4y - xk.y, sf0, cf0, sy0, cy0, y4x, mx);
-        if (!(mx <= kRotMax)) {  // a step too long for the small-angle turns
-          d2 = dg_derivs32(piA, t1.x, b1, y2x, y2y);
-          const float z3x = fmaf(h2, d2.u0, xk.x), z3y = fmaf(h2, d2.u1, xk.y);
-          d3 = dg_derivs32(piA, t1.x, b1, z3x, z3y);
-          d4 = dg_derivs32(piA, t2.x, b2, fmaf(h, d3.u0, xk.x), fmaf(h, d3.u1, xk.y));
+      auto reverse = [&](auto check) {
+        constexpr bool CHECK = decltype(check)::value;
+#pragma unroll 2
+        for (int k = k1 - 1; k >= k0; --k) {
+          const float2 xk = states[(k - k0) * blockDim.x + threadIdx.x];
+          const int m = 2 * (k - k0);
+          const float4 t0 = tab[m], t1 = tab[m + 1], t2 = tab[m + 2];
+          const float b0 = fmaf(-2.f, t0.x, 1.f);
+          // stage points (float); stages two to four turn stage one's sines and cosines
+          float2 sn, cs;
+          fsincospi(fmaf(t0.x, xk.x, b0) * xk.x, sn.x, cs.x);
+          fsincospi(xk.y, sn.y, cs.y);
+          const float e1 = fmaf(2.0f, xk.x, -2.0f), g0 = xk.x * (xk.x - 2.0f);
+          const DgStage d1 = dg_stage(sn.x, cs.x, sn.y, cs.y, fmaf(2.0f * t0.x, xk.x, b0), e1);
+          const float dg1 = (t1.x - t0.x) * g0, dg2 = (t2.x - t0.x) * g0;
+          float mx = 0.0f;
+          DgStage d2 = dg_stage_rot<CHECK>(t1.x, e1, dg1, a.hs[0][0] * d1.scy, a.hs_pi[0] * (d1.csy * d1.fx), sn, cs, mx);
+          DgStage d3 = dg_stage_rot<CHECK>(t1.x, e1, dg1, a.hs[0][0] * d2.scy, a.hs_pi[0] * (d2.csy * d2.fx), sn, cs, mx);
+          DgStage d4 = dg_stage_rot<CHECK>(t2.x, e1, dg2, a.hs[0][1] * d3.scy, a.hs_pi[1] * (d3.csy * d3.fx), sn, cs, mx);
+          if constexpr (CHECK) {
+            if (!(mx <= kRotMax)) {  // a step too long for the small-angle turns
+              const float b1 = fmaf(-2.f, t1.x, 1.f), b2 = fmaf(-2.f, t2.x, 1.f);
+              auto at = [&](const DgStage& d, int f, float c, float b) {
+                return dg_stage_full(c, b, fmaf(a.hs[0][f], d.scy, xk.x), fmaf(a.hs[1][f], d.csy * d.fx, xk.y));
+              };
+              d2 = at(d1, 0, t1.x, b1);
+              d3 = at(d2, 0, t1.x, b1);
+              d4 = at(d3, 1, t2.x, b2);
+            }
+          }
+          // the stage adjoints kb, the accumulated xb and lambda carry (x, y) as paired lanes
+          const float2 lam = make_float2(lam0, lam1);
+          float2 kb1 = mul2(f2(h6), lam), kb2 = mul2(f2(h3), lam), kb3 = kb2;
+          const float2 kb4 = kb1;
+          float2 xb = lam;
+          float2 yb = dg_reverse(d4, kb4, t2, piA, pi2A, s0, s1, s2);
+          xb = add2(xb, yb); kb3 = fma2(f2(h), yb, kb3);
+          yb = dg_reverse(d3, kb3, t1, piA, pi2A, s0, s1, s2);
+          xb = add2(xb, yb); kb2 = fma2(f2(h2), yb, kb2);
+          yb = dg_reverse(d2, kb2, t1, piA, pi2A, s0, s1, s2);
+          xb = add2(xb, yb); kb1 = fma2(f2(h2), yb, kb1);
+          yb = dg_reverse(d1, kb1, t0, piA, pi2A, s0, s1, s2);
+          const float2 ln = add2(xb, yb);
+          lam0 = ln.x;
+          lam1 = ln.y;
         }
-        // the stage adjoints kb, the accumulated xb and lambda carry (x, y) as paired lanes
-        const float2 lam = make_float2(lam0, lam1);
-        float2 kb1 = mul2(f2(h6), lam), kb2 = mul2(f2(h3), lam), kb3 = kb2;
-        const float2 kb4 = kb1;
-        float2 xb = lam;
-        auto stage = [&](const DgDer& d, float2 kb, const float4& tc) -> float2 {
-          const float2 yb = make_float2(fmaf(-d.j11, kb.x, d.j10 * kb.y), fmaf(d.j01, kb.x, d.j11 * kb.y));
-          const float qk = fmaf(d.q0, kb.x, d.q1 * kb.y);
-          s0 = fmaf(d.pA0, kb.x, fmaf(d.pA1, kb.y, s0));
-          s1 = fmaf(tc.z, qk, s1);
-          s2 = fmaf(eps * tc.w, qk, s2);
-          return yb;
-        };
-        float2 yb = stage(d4, kb4, t2);
-        xb = add2(xb, yb); kb3 = fma2(f2(h), yb, kb3);
-        yb = stage(d3, kb3, t1);
-        xb = add2(xb, yb); kb2 = fma2(f2(h2), yb, kb2);
-        yb = stage(d2, kb2, t1);
-        xb = add2(xb, yb); kb1 = fma2(f2(h2), yb, kb1);
-        yb = stage(d1, kb1, t0);
-        const float2 ln = add2(xb, yb);
-        lam0 = ln.x;
-        lam1 = ln.y;
-      }
+      };
+      if (safe)  // every angle within kRotMax (dg_node_safe)
+        reverse(std::false_type{});
+      else
+        reverse(std::true_type{});
       th0 += kPi * (double)s0;  // the pA terms are du/dA / pi
       th1 += (double)s1;
       th2 += (double)s2;
@@ -350,7 +356,7 @@ BwLayout bw_layout(int64_t n) {
   off += align256(sizeof(double) * 5 * (size_t)(n > 0 ? n : 1));
   L.phibar = off;
   off += align256(sizeof(float) * 2 * (size_t)(n > 0 ? n : 1));
-  L.nblocks = (int)((n + kAdjBlock - 1) / kAdjBlock);
+  L.nblocks = (int)((n + kAdjBlockMin - 1) / kAdjBlockMin);
   L.partial = off;
   off += align256(sizeof(double) * 3 * (size_t)(L.nblocks > 0 ? L.nblocks : 1));
   L.total = off;
@@ -358,12 +364,12 @@ BwLayout bw_layout(int64_t n) {
 }
 
 template <int PREC, int OUT>
-int launch_adjoint_rk4(const AdvArgs& a, const float* phibar, double* partial, int nblocks, size_t smem,
+int launch_adjoint_rk4(const AdvArgs& a, const float* phibar, double* partial, int nblocks, int block, size_t smem,
                        cudaStream_t s) {
   if (smem > 48 * 1024)
     FTLE_CUDA_CHECK(cudaFuncSetAttribute(k_adjoint_rk4<PREC, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem));
-  k_adjoint_rk4<PREC, OUT><<<nblocks, kAdjBlock, smem, s>>>(a, phibar, partial);
+  k_adjoint_rk4<PREC, OUT><<<nblocks, block, smem, s>>>(a, phibar, partial);
   FTLE_LAUNCH_CHECK("k_adjoint_rk4 launch");
   return FTLE_OK;
 }
@@ -429,13 +435,17 @@ int ftle_backward(const ftle_mesh* mesh, const ftle_flow* flow, double t0, doubl
   a.ckpt = const_cast<void*>(checkpoints);
   a.ckpt_every = ckpt_every;
   a.ckpt_stride_bytes = (int64_t)ftle_checkpoint_bytes(mesh->dim, mesh->n_nodes, precision);
-  const size_t smem = sizeof(float4) * (size_t)(2 * ckpt_every + 1) + sizeof(float2) * (size_t)ckpt_every * kAdjBlock;
+  // segments of up to 50 steps leave room for four blocks of 128 threads per SM, 512 x 256 nodes at
+  // T = 5, segments of 50 steps: 850 us, blocks of 64 threads 868-885, of 32 900
+  const int block = ckpt_every <= 50 ? kAdjBlock : kAdjBlockMin;
+  const int nblocks = (int)((mesh->n_nodes + block - 1) / block);
+  const size_t smem = sizeof(float4) * (size_t)(2 * ckpt_every + 1) + sizeof(float2) * (size_t)ckpt_every * block;
   if (precision == FTLE_PREC_FP32C)
-    rc = launch_adjoint_rk4<P32C, O32PAIR>(a, phibar, partial, W.nblocks, smem, s);
+    rc = launch_adjoint_rk4<P32C, O32PAIR>(a, phibar, partial, nblocks, block, smem, s);
   else
-    rc = launch_adjoint_rk4<P32, O32>(a, phibar, partial, W.nblocks, smem, s);
+    rc = launch_adjoint_rk4<P32, O32>(a, phibar, partial, nblocks, block, smem, s);
   if (rc) return rc;
-  k_sum_partials<<<1, 256, 0, s>>>(partial, W.nblocks, dL_dparams);
+  k_sum_partials<<<1, 256, 0, s>>>(partial, nblocks, dL_dparams);
   FTLE_LAUNCH_CHECK("k_sum_partials launch");
   return FTLE_OK;
 }
