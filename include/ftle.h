@@ -168,11 +168,13 @@ typedef struct ftle_options {
                              when an index is out of range.  The check synchronises the stream
                              once per mesh (it reads its counters back), so it is off by default;
                              ftle_compute_host always runs it. */
-  int32_t grad_staging;   /* float gradient of compensated flowmaps: 0 brings each tile's
+  int32_t grad_staging;   /* float gradient: 0 brings each tile's
                              neighbour indices into shared memory by bulk copies (TMA) one tile
                              ahead of the computation (the fixed-width list: width 6 in 2D or 14
                              in 3D, n_nodes a multiple of 4, ell_idx 16-byte aligned; CSR rows:
-                             col_idx 16-byte aligned), 1 reads the indices with plain loads.
+                             col_idx 16-byte aligned; flowmaps other than compensated ones with
+                             float coordinates: 3D CSR rows only), 1 reads the indices with
+                             plain loads.
                              Same results either way. */
   int32_t abc_refresh;    /* compensated ABC advection with the unchecked step (ftle_rotation_bounds
                              .unchecked): stage one's sines and cosines of the state are evaluated

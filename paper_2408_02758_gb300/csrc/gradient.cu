@@ -170,10 +170,14 @@ __global__ void __launch_bounds__(kStageTile) k_grad_f32_ell_staged(GradArgs a) 
 // node reads the few indices past that end (and every index of a stretch longer than a stage) from
 // global memory.  The per-node arithmetic and the neighbour order are grad_node_f32_rec's (same
 // results bit for bit).  The copy stays inside [0, nnz) whatever row_ptr holds; the gathers trust
-// the indices as the plain kernel does.
+// the indices as the plain kernel does.  Without records (plain float flowmaps, double coordinates) a
+// neighbour is 2 DIM scattered loads, as in grad_node_f32; the kernel waits for them (long_scoreboard,
+// 59 % issue), so four neighbours' loads go out together.  160^3 nodes, plain float, the whole gradient
+// call: 227 us with plain index loads, 209 staged, 200 with the four; in 2D (2048 x 1024) staging gains
+// 2 % at best and loses as much on smaller meshes, so those rows stay with the plain kernel.
 constexpr int kCsrStageInts = 16 * kStageTile;  // indices per stage: 16 per node of a full tile
 
-template <int DIM>
+template <int DIM, int PL, typename CT, bool REC>
 __global__ void __launch_bounds__(kStageTile) k_grad_f32_csr_staged(GradArgs a) {
   constexpr int T = kStageTile;
   __shared__ __align__(128) int32_t s_idx[2][kCsrStageInts];
@@ -249,12 +253,18 @@ __global__ void __launch_bounds__(kStageTile) k_grad_f32_csr_staged(GradArgs a) 
     }
     bool flag = false;
     if (i < n) {
-      float xi[DIM], hi_[DIM], li[DIM];
       float m[DIM * (DIM + 1) / 2] = {}, b[DIM * DIM] = {};
-      load_record<DIM>(a.rec, i, xi, hi_, li);
-      for (int e = rs; e < re; ++e) {
-        const int j = (e >= lo && e < hi) ? s_idx[stage][e - lo] : ld_index(a.col_idx + e);
-        grad_accumulate_rec<DIM>(a.rec, j, xi, hi_, li, m, b);
+      auto index = [&](int e) { return (e >= lo && e < hi) ? s_idx[stage][e - lo] : ld_index(a.col_idx + e); };
+      if constexpr (REC) {
+        float xi[DIM], hi_[DIM], li[DIM];
+        load_record<DIM>(a.rec, i, xi, hi_, li);
+        for (int e = rs; e < re; ++e) grad_accumulate_rec<DIM>(a.rec, index(e), xi, hi_, li, m, b);
+      } else {
+        CT xi[DIM];
+        float2 pi[DIM];
+        grad_load_self<DIM, PL, CT>(a, i, xi, pi, m, b);
+#pragma unroll 4
+        for (int e = rs; e < re; ++e) grad_accumulate<DIM, PL, CT>(a, index(e), xi, pi, m, b);
       }
       mbar_arrive(&s_empty[stage]);
       flag = grad_finish_f32<DIM>(a, i, re - rs, m, b);
@@ -360,19 +370,19 @@ static bool grad_f32_ell_staged(const GradArgs& a, cudaStream_t s) {
   return true;
 }
 
-// The staged CSR kernel applies to records over any rows (col_idx 16-byte aligned).
-template <int DIM>
+// The staged CSR kernel applies to any rows (col_idx 16-byte aligned).
+template <int DIM, int PL, typename CT, bool REC>
 static bool grad_f32_csr_staged(const GradArgs& a, cudaStream_t s) {
   if (!a.staged || a.nnz <= 0 || ((uintptr_t)a.col_idx & 15)) return false;
   const int64_t tiles = (a.n + kStageTile - 1) / kStageTile;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grad_f32_csr_staged<DIM>, kStageTile, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grad_f32_csr_staged<DIM, PL, CT, REC>, kStageTile, 0) !=
           cudaSuccess ||
       per_sm < 1)
     per_sm = 1;
   const int sms = device_sm_count() > 0 ? device_sm_count() : 1;
   const int64_t cap = (int64_t)sms * per_sm;
-  k_grad_f32_csr_staged<DIM><<<(int)(tiles < cap ? tiles : cap), kStageTile, 0, s>>>(a);
+  k_grad_f32_csr_staged<DIM, PL, CT, REC><<<(int)(tiles < cap ? tiles : cap), kStageTile, 0, s>>>(a);
   return true;
 }
 
@@ -422,12 +432,18 @@ static void grad_f32_dispatch(bool coord64, const GradArgs& a, int grid, int blo
       grad_f32_ell_dispatch<DIM, PL, float, false>(a, grid, block, s);
   } else if (rec) {
     if constexpr (PL == PHI32PAIR) {
-      if (grad_f32_csr_staged<DIM>(a, s)) return;
+      if (grad_f32_csr_staged<DIM, PL, float, true>(a, s)) return;
+      k_grad_f32<DIM, PL, float, true><<<grid, block, 0, s>>>(a);
     }
-    k_grad_f32<DIM, PL, float, true><<<grid, block, 0, s>>>(a);
   } else if (coord64) {
+    if constexpr (DIM == 3) {
+      if (grad_f32_csr_staged<DIM, PL, double, false>(a, s)) return;
+    }
     k_grad_f32<DIM, PL, double, false><<<grid, block, 0, s>>>(a);
   } else {
+    if constexpr (DIM == 3) {
+      if (grad_f32_csr_staged<DIM, PL, float, false>(a, s)) return;
+    }
     k_grad_f32<DIM, PL, float, false><<<grid, block, 0, s>>>(a);
   }
 }

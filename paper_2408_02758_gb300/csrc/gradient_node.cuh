@@ -106,17 +106,23 @@ __device__ __forceinline__ void grad_moments(const float* dx, const float* dp, f
     for (int c = 0; c < DIM; ++c) b[r * DIM + c] = fmaf(dp[r], dx[c], b[r * DIM + c]);
 }
 
-// Float moments of one neighbour j read from the coordinate and flowmap arrays.
+// Float moments of one neighbour j read from the coordinate and flowmap arrays (a 32-bit offset from
+// each array's start: one address operation a load).
 template <int DIM, int PL, typename CT>
-__device__ __forceinline__ void grad_accumulate(const GradArgs& a, int64_t j, const CT* xi, const float2* pi,
+__device__ __forceinline__ void grad_accumulate(const GradArgs& a, int64_t j64, const CT* xi, const float2* pi,
                                                 float* m, float* b) {
-  const int64_t n = a.n;
+  const int32_t j = (int32_t)j64;
   float dx[DIM], dp[DIM];
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
-    dx[d] = (float)(ldc<CT>(a.coords, d * n + j) - xi[d]);
-    const float2 pj = ld_phi32<PL>(a.phi, d * n + j);
-    dp[d] = (pj.x - pi[d].x) + (pj.y - pi[d].y);
+    const CT* c = reinterpret_cast<const CT*>(a.coords) + d * a.n;
+    dx[d] = (float)(__ldg(c + j) - xi[d]);
+    float2 pj;
+    if constexpr (PL == PHI32PAIR)
+      pj = __ldg(reinterpret_cast<const float2*>(a.phi) + d * a.n + j);
+    else
+      pj = make_float2(__ldg(reinterpret_cast<const float*>(a.phi) + d * a.n + j), 0.f);
+    dp[d] = PL == PHI32PAIR ? (pj.x - pi[d].x) + (pj.y - pi[d].y) : pj.x - pi[d].x;
   }
   grad_moments<DIM>(dx, dp, m, b);
 }
