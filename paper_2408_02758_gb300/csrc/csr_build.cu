@@ -40,7 +40,9 @@ __device__ __forceinline__ void load_element(const int32_t* __restrict__ elems, 
 
 // One returned atomic and one store per element and vertex, the element's number; appending the other
 // vertices instead (12 atomics and stores a tetrahedron, or 4 atomics and 12 stores) is bound by
-// the scattered accesses: 674 and 420 us for 5.14 M tetrahedra of 96^3 nodes, 223 now.  Element numbers fit
+// the scattered accesses: 674 and 420 us for 5.14 M tetrahedra of 96^3 nodes, 221 now (the eight scattered
+// accesses of an element, a line each, take the first-level caches about 140).  One atomic for a warp's equal
+// vertices (match_any) loses 10-20 % on meshes whose elements come cell by cell.  Element numbers fit
 // a slot up to 2^32 elements; beyond that (WIDE) the vertices themselves are appended.
 template <bool WIDE>
 __global__ void __launch_bounds__(256) k_elem_pairs(int64_t n_elem, int v, const int32_t* __restrict__ elems,
@@ -88,24 +90,46 @@ __global__ void __launch_bounds__(256) k_elem_pairs(int64_t n_elem, int v, const
 }
 
 // Rows of a block of kRowBlock nodes, one per thread: the other vertices of the node's elements go
-// one by one into a hash table of kRowSlots places in shared memory (a column per thread, so the
-// lanes of a warp never share a bank); the distinct ones are then sorted in the column's head.  A
-// tetrahedral row has ~72 raw and 14 distinct entries, so most raw ones cost one probe: for 96^3
-// nodes 391 us, against 419 with halving into a sorted list and 7545 with the raw ones sorted in
-// global memory (72^2 / 4 moves a row).  What bounds it now is instruction issue with 14 of 32
-// lanes active on average (probing and sorting diverge).  The block's lists are then packed, in node order, from the start
-// of the block's slots (their place in row_ptr is then the block's start plus an offset scanned
-// here, and their copy into col_idx is one contiguous stretch).  A row with more than kRowList
-// distinct entries is built where its slots lie instead, and its block's rows all stay in their
-// own slots (kBlockSpread in the block's total).  The total takes the place of the block's first
+// one by one into a hash table in shared memory (kRowSlots places in buckets of two, one load a probe;
+// a column per thread), the next four elements' numbers loading meanwhile.  A tetrahedral row has 72 raw
+// and 14 distinct entries, so most raw ones cost one probe.  The distinct ones are sorted in registers,
+// the same exchanges in every lane: by a network of 8 or 16 behind a move to the column's head when the
+// longest of the warp's rows fits it, of 32 from the table as it lies otherwise.  96^3 nodes: 182 us;
+// 233 with the network of 32 throughout, 391 with one place a probe and an insertion sort in the
+// column (14 of 32 lanes active on average; 23 with the network of 32), 7545 with the raw entries sorted in
+// global memory (72^2 / 4 moves a row).  What bounds it now is the first-level cache, where each lane's
+// element is a line of its own.  The block's lists are packed in shared memory and go, in node
+// order, to the start of the block's slots (their place in row_ptr is then the block's start plus an
+// offset scanned here, and their copy into col_idx is one contiguous stretch).  A row with more than
+// kRowList distinct entries is built where its slots lie instead, and its block's rows all stay in
+// their own slots (kBlockSpread in the block's total).  The total takes the place of the block's first
 // two raw counts, which this block alone reads.
 constexpr int kRowBlock = 128;
-constexpr int kRowSlots = 32;  // a power of two
+constexpr int kRowSlots = 32;  // in buckets of two
 constexpr int kRowList = 28;   // distinct entries the table takes
 constexpr int64_t kBlockSpread = (int64_t)1 << 62;
 
 __device__ __forceinline__ int64_t* block_total(int32_t* raw, int64_t block) {
   return reinterpret_cast<int64_t*>(raw + block * kRowBlock);
+}
+
+// Sorts N values in registers (Batcher's odd-even merge sort: 19, 63 and 191 exchanges for 8, 16 and 32,
+// the same for every lane).
+template <int N>
+__device__ __forceinline__ void sort_net(uint32_t* r) {
+#pragma unroll
+  for (int p = 1; p < N; p <<= 1)
+#pragma unroll
+    for (int k = p; k >= 1; k >>= 1)
+#pragma unroll
+      for (int j = k % p; j + k < N; j += 2 * k)
+#pragma unroll
+        for (int i = 0; i < k; ++i)
+          if (i + j + k < N && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+            const uint32_t lo = min(r[i + j], r[i + j + k]), hi = max(r[i + j], r[i + j + k]);
+            r[i + j] = lo;
+            r[i + j + k] = hi;
+          }
 }
 
 // Inclusive scan over the warp.
@@ -140,39 +164,40 @@ __device__ __forceinline__ int64_t block_scan(int64_t v, int64_t& total) {
 }
 
 template <bool WIDE>
-__global__ void __launch_bounds__(kRowBlock) k_row_unique(int64_t n_nodes, int v, const int32_t* __restrict__ elems,
+__global__ void __launch_bounds__(kRowBlock, 9) k_row_unique(int64_t n_nodes, int v, const int32_t* __restrict__ elems,
                                                           int cap, int32_t* __restrict__ slots,
                                                           int32_t* __restrict__ raw, int32_t* __restrict__ row_ptr,
                                                           CsrBuildFlags* flags) {
-  __shared__ int32_t s_list[kRowSlots][kRowBlock];
+  __shared__ __align__(16) int2 s_tab[kRowSlots / 2][kRowBlock];
   const bool vec = v == 4 && ((uintptr_t)elems & 15) == 0;
   const int t = threadIdx.x;
   const int64_t first = (int64_t)blockIdx.x * kRowBlock, i = first + t;
   int32_t* row = slots + i * cap;
   const int k = i < n_nodes ? max(0, min(raw[i], cap)) : 0;
-  // the raw neighbours of slot entry x: up to 3 of an element's vertices, or x itself
+  // the raw neighbours of slot entry x: up to 3 of an element's vertices, or x itself; -1: none
+  constexpr int E = WIDE ? 1 : 3;
   auto expand = [&](int32_t x, int32_t* nb) {
-    int c = 0;
     if constexpr (WIDE) {
-      nb[c++] = x;
+      nb[0] = x;
     } else {
       int32_t vert[4];
       load_element(elems, v, vec, (int64_t)(uint32_t)x, vert);
+      int32_t last = vert[3] == (int32_t)i ? -1 : vert[3];  // takes the place of the node itself
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        nb[q] = q < v && vert[q] != (int32_t)i ? vert[q] : -1;  // -1: none
-      c = 4;
+      for (int q = 0; q < 3; ++q) {
+        const bool self = vert[q] == (int32_t)i;
+        nb[q] = self ? last : vert[q];
+        last = self ? -1 : last;
+      }
     }
-    return c;
   };
-  constexpr int E = WIDE ? 1 : 4;
   int u = 0, n_raw = 0;
   bool fits = true;
-  static_assert(kRowSlots == 32 && kRowList < kRowSlots, "the hash keeps five bits and never fills the table");
+  static_assert(kRowSlots == 32 && kRowList < kRowSlots, "the hash keeps four bits and never fills the table");
 #pragma unroll
-  for (int h = 0; h < kRowSlots; ++h) s_list[h][t] = -1;
-  for (int a0 = 0; a0 < k && fits; a0 += 4) {
-    int32_t x[4], nb[4][E];
+  for (int h = 0; h < kRowSlots / 2; ++h) s_tab[h][t] = make_int2(-1, -1);
+  int32_t x[4];
+  auto load4 = [&](int a0) {
     if ((cap & 3) == 0) {  // the row starts on 16 bytes: one load for four entries
       const int4 r = *reinterpret_cast<const int4*>(row + a0);
       x[0] = r.x, x[1] = r.y, x[2] = r.z, x[3] = r.w;
@@ -180,41 +205,62 @@ __global__ void __launch_bounds__(kRowBlock) k_row_unique(int64_t n_nodes, int v
 #pragma unroll
       for (int q = 0; q < 4; ++q) x[q] = a0 + q < k ? row[a0 + q] : 0;
     }
+  };
+  if (k > 0) load4(0);
+  for (int a0 = 0; a0 < k && fits; a0 += 4) {
+    int32_t nb[4][E];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {  // four elements' loads in flight
 #pragma unroll
       for (int r = 0; r < E; ++r) nb[q][r] = -1;
       if (a0 + q < k) expand(x[q], nb[q]);
     }
+    if (a0 + 4 < k) load4(a0 + 4);
 #pragma unroll
     for (int q = 0; q < 4 * E; ++q) {
       const int32_t y = nb[q / E][q % E];
       if (y < 0 || !fits) continue;
       ++n_raw;
-      int h = (int)(((uint32_t)y * 0x9E3779B1u) >> 27);  // 5 bits: kRowSlots
-      int32_t z = s_list[h][t];
-      while (z != y && z >= 0) {  // kRowList < kRowSlots: an empty place is always met
-        h = (h + 1) & (kRowSlots - 1);
-        z = s_list[h][t];
+      int h = (int)(((uint32_t)y * 0x9E3779B1u) >> 28);  // 4 bits: kRowSlots / 2
+      int2 z = s_tab[h][t];
+      while (z.x != y && z.y != y && z.y >= 0) {  // kRowList < kRowSlots: an empty place is always met
+        h = (h + 1) & (kRowSlots / 2 - 1);
+        z = s_tab[h][t];
       }
-      if (z == y) continue;
-      if (u == kRowList) {
-        fits = false;
-        continue;
-      }
-      s_list[h][t] = y;
-      ++u;
+      const bool fresh = z.x != y && z.y != y;
+      fits = !fresh || u < kRowList;
+      if (fresh && fits) reinterpret_cast<int32_t*>(&s_tab[h][t])[z.x < 0 ? 0 : 1] = y;
+      u += fresh && fits;
     }
   }
-  if (fits) {  // the distinct entries, sorted into the head of the column
+  uint32_t list[kRowSlots];  // the distinct entries, sorted; empty places (all ones) come last
+  const int u_max = __reduce_max_sync(0xffffffffu, u);  // of the warp's rows
+  if (u_max <= 16) {  // the entries to the head of the column, and a smaller network
+    int32_t* col = reinterpret_cast<int32_t*>(&s_tab[0][t]);
+    auto place = [](int w) { return (w >> 1) * (2 * kRowBlock) + (w & 1); };
     int w = 0;
-    for (int h = 0; w < u; ++h) {
-      const int32_t y = s_list[h][t];
-      if (y < 0) continue;
-      int b = w++;
-      for (; b > 0 && s_list[b - 1][t] > y; --b) s_list[b][t] = s_list[b - 1][t];
-      s_list[b][t] = y;
+#pragma unroll
+    for (int h = 0; h < kRowSlots / 2; ++h) {
+      const int2 z = s_tab[h][t];
+      if (z.x >= 0) col[place(w++)] = z.x;
+      if (z.y >= 0) col[place(w++)] = z.y;
     }
+#pragma unroll
+    for (int a = 0; a < 16; ++a) list[a] = a < w ? (uint32_t)col[place(a)] : ~0u;
+#pragma unroll
+    for (int a = 16; a < kRowSlots; ++a) list[a] = ~0u;
+    if (u_max <= 8)
+      sort_net<8>(list);
+    else
+      sort_net<16>(list);
+  } else {
+#pragma unroll
+    for (int h = 0; h < kRowSlots / 2; ++h) {
+      const int2 z = s_tab[h][t];
+      list[2 * h] = (uint32_t)z.x;
+      list[2 * h + 1] = (uint32_t)z.y;
+    }
+    sort_net<kRowSlots>(list);
   }
   if (!fits) {
     // The row's entries move to the end of its slots and the sorted list grows from the start: it
@@ -226,8 +272,9 @@ __global__ void __launch_bounds__(kRowBlock) k_row_unique(int64_t n_nodes, int v
     for (int a = k - 1; a >= 0; --a) row[base + a] = row[a];
     for (int a = 0; a < k; ++a) {
       int32_t nb[E];
-      const int c = expand(row[base + a], nb), room = base + a + 1;
-      for (int r = 0; r < c; ++r) {
+      const int room = base + a + 1;
+      expand(row[base + a], nb);
+      for (int r = 0; r < E; ++r) {
         const int32_t y = nb[r];
         if (y < 0) continue;
         ++n_raw;
@@ -254,34 +301,51 @@ __global__ void __launch_bounds__(kRowBlock) k_row_unique(int64_t n_nodes, int v
   int64_t total;
   const int64_t off = block_scan<kRowBlock / 32>(u, total) - u;
   if (i < n_nodes) row_ptr[i] = (int32_t)off;
-  if (fits) {
-    int32_t* dst = spread ? row : slots + first * cap + off;
-    for (int a = 0; a < u; ++a) dst[a] = s_list[a][t];
+  if (spread) {
+    if (fits) {
+#pragma unroll
+      for (int a = 0; a < kRowList; ++a)
+        if (a < u) row[a] = (int32_t)list[a];
+    }
+  } else {  // packed in shared memory first (the tables have been read), then written in order
+    int32_t* s_pack = reinterpret_cast<int32_t*>(s_tab);
+#pragma unroll
+    for (int a = 0; a < kRowList; ++a)
+      if (a < u) s_pack[off + a] = (int32_t)list[a];
+    __syncthreads();
+    for (int a = t; a < (int)total; a += kRowBlock) slots[first * cap + a] = s_pack[a];
   }
   if (t == 0) *block_total(raw, blockIdx.x) = total | (spread ? kBlockSpread : 0);
 }
 
-// Exclusive scan of the blocks' totals in place, by one block: each thread sums its share, the
-// shares are scanned, and the totals are replaced by the blocks' starts.
+// Exclusive scan of the blocks' totals in place, by one block, which replaces them by the blocks' starts:
+// kSumEach totals a thread at a time, all loaded before the first is used (the chain of loads is what
+// bounds this: 12 us for 6912 totals, 19 when each was read before the next).
 constexpr int kSumThreads = 1024;
+constexpr int kSumEach = 8;
 
 __global__ void __launch_bounds__(kSumThreads) k_scan_sums(int64_t nb, int64_t n_nodes, int32_t* __restrict__ raw,
                                                            int32_t* __restrict__ row_ptr, CsrBuildFlags* flags) {
-  const int64_t per = (nb + kSumThreads - 1) / kSumThreads;
-  const int64_t lo = min(nb, threadIdx.x * per), hi = min(nb, lo + per);
-  int64_t sum = 0;
-#pragma unroll 4
-  for (int64_t b = lo; b < hi; ++b) sum += *block_total(raw, b) & ~kBlockSpread;
-  int64_t total;
-  int64_t run = block_scan<kSumThreads / 32>(sum, total) - sum;
-  for (int64_t b = lo; b < hi; ++b) {
-    const int64_t v = *block_total(raw, b);
-    *block_total(raw, b) = run | (v & kBlockSpread);
-    run += v & ~kBlockSpread;
+  int64_t before = 0;
+  for (int64_t b0 = 0; b0 < nb; b0 += kSumThreads * kSumEach) {
+    const int64_t lo = b0 + (int64_t)threadIdx.x * kSumEach;
+    int64_t v[kSumEach], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kSumEach; ++q) v[q] = lo + q < nb ? *block_total(raw, lo + q) : 0;
+#pragma unroll
+    for (int q = 0; q < kSumEach; ++q) sum += v[q] & ~kBlockSpread;
+    int64_t total;
+    int64_t run = before + block_scan<kSumThreads / 32>(sum, total) - sum;
+#pragma unroll
+    for (int q = 0; q < kSumEach; ++q) {
+      if (lo + q < nb) *block_total(raw, lo + q) = run | (v[q] & kBlockSpread);
+      run += v[q] & ~kBlockSpread;
+    }
+    before += total;
   }
   if (threadIdx.x == 0) {
-    flags->nnz = (unsigned long long)total;
-    row_ptr[n_nodes] = (int32_t)total;
+    flags->nnz = (unsigned long long)before;
+    row_ptr[n_nodes] = (int32_t)before;
   }
 }
 
