@@ -40,21 +40,22 @@ FLUSH_BYTES = 320 << 20
 # Algorithmic FP32 flops of one compensated RK4 step per node as the kernels take it (FMA = 2
 # flops; one sincospi or sincos counted as 20 flops: argument reduction plus degree-7/8 minimax
 # polynomials; a small-angle rotation of a (sin, cos) pair 15).
-#   double gyre: stage one 74 (error-free f 17, two sincospi 40, first-order corrections 10,
-#                slope and velocity 7), per-step terms 6, stage two 39 (two rotations without
-#                the fourth-order cosine term 26, angles 7, slope 2, increment 1, velocity 3),
-#                stage four 43 (two rotations 30, the same 13), stage three 27 (angles and
-#                their differences 11, four first-order turns 12, slope and velocity 4), update
-#                22 (the step scale in two parts)
-#   ABC:         stage one 87 when evaluated afresh (three compensated sincos 78, increments 9)
-#                or 24 when carried from the previous step (stage four's three pairs turned to
-#                first order by the rest of the step's increment 15, increments 9; fresh once
-#                every abc_refresh = 8 steps), stage two 48 (three rotations without the
-#                fourth-order cosine term 39, increments 9), stage three 24 (three first-order
-#                turns 15, increments 9), stage four 54 (three rotations 45, increments 9) or 48
-#                on a carried step (its rotations without that term, as at stage two), update 27
+#   double gyre: stage one from the carried pairs 11, per-step terms 11, stage two 37 (two turns
+#                without the fourth-order cosine term, their corrections kept apart 26, angles 6,
+#                velocity 5), stage three 25 (angles and their differences 8, four first-order
+#                turns 12, velocity 5), stage four 45 (two turns onto the corrections 34, angles
+#                and slope 8, velocity 3), the weighted sum 8, the pairs on to the next step 17,
+#                update 14 (the step scale in two parts); every 16 steps the pairs afresh 65 and
+#                once in between the corrections joined to them 12
+#   ABC:         increments 9 each at stages one to three, stages two and four 39 each (three
+#                rotations without the fourth-order cosine term), stage three 18 (three
+#                first-order turns), stage four's increments and the weighted sum 21; the pairs on
+#                to the next step 18 on seven steps of eight, afresh 78 on the eighth (three
+#                compensated sincos, every abc_refresh = 8 steps); the state's update 27 on every
+#                fourth step and the sum of the increments 3 on the others, 9 a step
 ABC_REFRESH = 8
-FLOPS_PER_POINT_STEP = {"dg": 211, "abc": 240 - (63 + 6) * (ABC_REFRESH - 1) / ABC_REFRESH}
+FLOPS_PER_POINT_STEP = {"dg": 168 + (65 + 12) / 16,
+                        "abc": 144 + (18 * (ABC_REFRESH - 1) + 78) / ABC_REFRESH + 9}
 
 
 def peak_fp32_tflops(sms: int, mhz: float) -> float:
@@ -648,7 +649,7 @@ def main():
         "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
         "data": "synthetic",
         "config": workload_config(w, world, layout_of(args)), "tuned": tuned or "defaults (--no-tune)",
-        "roofline": {"kernel": "k_advect (RK4 flowmap)", "bound": "alu", "achieved": achieved, "peak": peak,
+        "roofline": {"kernel": "advection (k_advect_abc, k_advect_dg: RK4 flowmap)", "bound": "alu", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak,
                      "peak_source": f"{sms} SMs x 128 FP32 lanes x 2 flops x {peaks.get('sm_max_mhz', 2070.0)} MHz "
                                     "(max SM clock of measured peaks)",

@@ -149,8 +149,9 @@ typedef struct ftle_options {
                              rank, conditioning and lambda_max - 1 < 0.01 checks remain). */
   int32_t advect_block;   /* threads per block of the advection kernel (multiple of 32) */
   int32_t advect_blocks_per_sm; /* blocks per SM the advection grid is sized for (default
-                                   8192 / advect_block; a block loops over node tiles while
-                                   the grid is smaller than the mesh) */
+                                   8192 / advect_block, for the kernels that take two nodes
+                                   per thread as many as even out over the SMs; a block loops
+                                   over node tiles while the grid is smaller than the mesh) */
   int32_t grad_block;     /* threads per block of the gradient kernel (multiple of 32) */
   int32_t grad_tile;      /* nodes per gradient tile (multiple of grad_block) */
   int32_t refine_lanes;   /* re-advection: active lanes per 32-thread block (1..32); fewer lanes
@@ -232,7 +233,8 @@ int ftle_advect(const ftle_mesh* mesh, const ftle_flow* flow, double t0, double 
  *   unchecked    1 when both bounds are within their limits, else 0;
  *   carried      ABC: 1 when the unchecked step also carries stage one's sines and cosines from
  *                step to step (ftle_options.abc_refresh > 1 asks for it), i.e. unchecked and
- *                angle_bound within 0.032 rad (with the same margin); else 0.
+ *                angle_bound within 0.032 rad (with the same margin); else 0.  (The compensated
+ *                double gyre carries its pairs under the same two conditions; this field stays 0.)
  * Flows without the rotated step (linear, saddle): unchecked = 0, both bounds +inf.
  * Host only (no device work).  Errors: FTLE_EINVAL (null flow or out, unknown kind, parameters
  * or dt not finite, dt = 0). */
@@ -380,8 +382,9 @@ int ftle_gradient_eig_noalloc(const ftle_mesh* mesh, const void* flowmap, int32_
 
 /* ---------------------------------------------------------------------------------- batched */
 
-/* Many independent problems of uneven size and horizon in one launch sequence: one persistent
- * advection kernel and one persistent gradient kernel walk a shared queue of (instance, tile)
+/* Many independent problems of uneven size and horizon in one launch sequence: a persistent
+ * advection kernel (one for the instances whose sines and cosines are carried from step to step, one for
+ * the rest, where there are both) and a persistent gradient kernel walk queues of (instance, tile)
  * items ordered longest-first (LPT), followed by the FP64 fix-up of flagged nodes.  All
  * instances share dt and precision (FP32 or FP32C); per-instance t0 = 0.
  *   meshes, flows, T  HOST arrays [n_inst] (mesh pointers inside are device pointers).

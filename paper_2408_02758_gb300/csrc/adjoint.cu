@@ -179,9 +179,9 @@ __device__ __forceinline__ void build_adj_table(const AdvArgs& a, float4* tab, i
   }
 }
 
-// Bound by instruction issue: the recomputed forward step and the reverse of four stages, with the segment's
-// states in shared memory (8 bytes a step and thread, so 16 to 20 warps per SM).  512 x 256 nodes,
-// T = 5, 500 steps: 850 us; 1002 with J^T and P^T formed apart and the angles checked at each stage.
+// Bound by the FP32 pipe (73 % busy) at the 13 warps per SM that registers and the segment's states in
+// shared memory (8 bytes a step and thread) leave: the recomputed forward step and the reverse of four
+// stages.  512 x 256 nodes, T = 5, 500 steps: 850 us; 1002 with J^T and P^T formed apart and the angles checked at each stage.
 template <int PREC, int OUT>
 __global__ void __launch_bounds__(kAdjBlock) k_adjoint_rk4(AdvArgs a, const float* __restrict__ phibar,
                                                            double* __restrict__ partial) {

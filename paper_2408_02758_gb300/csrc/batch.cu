@@ -1,7 +1,8 @@
 // Batched FTLE: many independent problems of uneven mesh size and horizon in one launch
 // sequence.  The host plans a queue of (instance, node range) items ordered longest-first (LPT:
 // cost = nodes x RK4 steps), persistent blocks pull items with one atomic per item, and the per
-// node arithmetic is the single-problem kernels' (rk4_step, grad_node_f32, grad_node_f64), so
+// node arithmetic is the single-problem kernels' (rk4_step, the carried steps' dg_walk and abc_walk on a
+// queue of their own, grad_node_f32, grad_node_f64), so
 // every instance's FTLE equals its single-problem result.  Nodes that need the FP64 path are kept
 // as (instance, node) pairs; their re-advection runs in float-float with per-lane time
 // coefficients (lanes of one warp may belong to different instances).  The sequence can be
